@@ -325,11 +325,23 @@ struct DftPfa {
 template <typename T, int DIR>
 struct Dft<T, 6, DIR> : DftPfa<T, 3, 2, DIR> {};
 template <typename T, int DIR>
+struct Dft<T, 9, DIR> : DftComposite<T, 3, 3, DIR> {};
+template <typename T, int DIR>
 struct Dft<T, 10, DIR> : DftPfa<T, 5, 2, DIR> {};
 template <typename T, int DIR>
 struct Dft<T, 12, DIR> : DftPfa<T, 4, 3, DIR> {};
 template <typename T, int DIR>
 struct Dft<T, 16, DIR> : DftComposite<T, 4, 4, DIR> {};
+template <typename T, int DIR>
+struct Dft<T, 15, DIR> : DftPfa<T, 5, 3, DIR> {};
+template <typename T, int DIR>
+struct Dft<T, 18, DIR> : DftPfa<T, 9, 2, DIR> {};
+template <typename T, int DIR>
+struct Dft<T, 20, DIR> : DftPfa<T, 5, 4, DIR> {};
+template <typename T, int DIR>
+struct Dft<T, 25, DIR> : DftComposite<T, 5, 5, DIR> {};
+template <typename T, int DIR>
+struct Dft<T, 27, DIR> : DftComposite<T, 9, 3, DIR> {};
 // register-resident lengths of the one-thread-per-line kernels
 template <typename T, int DIR>
 struct Dft<T, 24, DIR> : DftPfa<T, 8, 3, DIR> {};

@@ -265,30 +265,55 @@ std::vector<CopyBlk> build_blocks(const psatd_plan_desc* d) {
 // ---------------------------------------------------------------------------
 namespace psatd {
 
-// Radix schedule: 8s first (4,4 instead of 8,2), then 4 / 2, 3s and 5s.
-bool radix_plan(int n, AxisPlan& ap) {
-  ap.n = n;
-  ap.npass = 0;
-  int e2 = 0, v = n;
-  while (v % 2 == 0) v /= 2, ++e2;
-  std::vector<int> r;
-  int n8 = e2 / 3, rem = e2 % 3;
-  if (rem == 1 && n8 > 0) {
-    --n8;
-    rem = 4;
-  }
-  for (int i = 0; i < n8; ++i) r.push_back(8);
-  if (rem == 4) r.push_back(4), r.push_back(4);
-  if (rem == 2) r.push_back(4);
-  if (rem == 1) r.push_back(2);
-  while (v % 5 == 0) v /= 5, r.push_back(5);
-  while (v % 3 == 0) v /= 3, r.push_back(3);
-  if (v != 1 || (int)r.size() > kMaxPass) return false;
-  for (size_t i = 0; i < r.size(); ++i) ap.radix[i] = (uint8_t)r[i];
-  ap.npass = (int)r.size();
-  return true;
+// Split n = r1 * r2 over the radices of the generic kernels: fewest operations
+// per point -- those of the two small DFTs (counted from the codelets: complex
+// sums, products and fused multiply-adds) and 4 per twiddle, of which coprime
+// radices need none (prime-factor maps) -- plus half an operation per unit of
+// imbalance, since the smaller radix leaves that many lanes without work.
+// Radices above 16 cost registers and are taken where nothing else divides n.
+bool line_plan(int n, AxisPlan& ap) {
+  static const struct {
+    int r;
+    double ops;
+  } kRadix[] = {{1, 0},    {2, 2},     {3, 4.67},   {4, 4},     {5, 7.2},    {6, 6.67},   {8, 7},
+                {9, 11.1}, {10, 9.2},  {12, 8.67},  {15, 11.9}, {16, 10.5},  {18, 13.1},  {20, 11.2},
+                {24, 11.7}, {25, 17},  {27, 18.5},  {30, 13.9}, {32, 13.5}};
+  auto gcd = [](int a, int b) {
+    while (b) {
+      const int t = a % b;
+      a = b;
+      b = t;
+    }
+    return a;
+  };
+  auto inverse = [](int a, int m) {   // a^-1 mod m (0 for m = 1)
+    for (int r = 0; r < m; ++r)
+      if ((a % m) * r % m == 1 % m) return r;
+    return 0;
+  };
+  const int64_t tw = ap.tw;
+  double best = 1e9;
+  for (const auto& a : kRadix)
+    for (const auto& b : kRadix) {
+      if (a.r * b.r != n) continue;
+      const int lo = std::min(a.r, b.r), hi = std::max(a.r, b.r);
+      const bool coprime = gcd(a.r, b.r) == 1;
+      const double cost = a.ops + b.ops + (coprime ? 0.0 : 4.0 * (a.r - 1) * (b.r - 1) / n) + 0.5 * hi / lo +
+                          (hi > 16 ? 100.0 : 0.0);
+      if (cost >= best) continue;
+      best = cost;
+      ap = AxisPlan{};
+      ap.n = n;
+      ap.r1 = a.r;
+      ap.r2 = b.r;
+      ap.wrap = coprime;
+      ap.a_in = coprime ? a.r : 1;
+      ap.a_out = coprime ? b.r * inverse(b.r, a.r) % n : 1;
+      ap.s_out = coprime ? a.r * inverse(a.r, b.r) % n : a.r;
+    }
+  ap.tw = tw;
+  return best < 1e9;
 }
-
 
 // Order-p staggered stencil weights (see tables.cu for their use):
 std::vector<double> stencil_alpha(int p, bool nodal) {
@@ -307,6 +332,12 @@ std::vector<double> stencil_alpha(int p, bool nodal) {
     a[l - 1] = v;
   }
   return a;
+}
+
+void column_tiles(std::vector<ColJob>& out, int box, int p0, int p1, int hx, int w) {
+  const int64_t total = (int64_t)(p1 - p0) * hx;
+  for (int64_t q = 0; q < total; q += w)
+    out.push_back({box, p0 + (int32_t)(q / hx), (int32_t)(q % hx), (int32_t)std::min<int64_t>(w, total - q)});
 }
 
 void set_thread_error(const char* msg) { g_thread_error = msg; }
@@ -329,8 +360,8 @@ struct psatd_plan {
 
   std::vector<BoxDev> hboxes;
   std::vector<ShapeDev> hshapes;
-  std::vector<RowJob> rows_all, rows_int;
-  std::vector<ColJob> ycols_all, ycols_int, zcols;           // every box (standalone FFTs)
+  std::vector<RowJob> rows_all;
+  std::vector<ColJob> ycols_all, zcols;                      // every box (standalone FFTs)
   std::vector<RowJob> g_rows, g_rows_int;                     // push, generic boxes
   std::vector<ColJob> g_ycols, g_ycols_int, g_zcols;
   std::vector<int2> plane_fwd, plane_inv;                     // push, fast boxes
@@ -379,7 +410,7 @@ struct psatd_plan {
 
   int64_t field_total = 0;  // elements per field buffer
   int64_t spec_total = 0;   // complex elements per spectrum slot
-  int smem_fx = 0, smem_y = 0, smem_z = 0, smem_zonly = 0, smem_ix = 0;
+  LineCfg cfg_fx, cfg_y, cfg_z, cfg_zonly, cfg_ix;   // generic kernels: launches that cover every box
   int smem_pf = 0, smem_pi = 0, smem_zf = 0;
   int smem_penx = 0, smem_penxi = 0, smem_penc = 0, smem_penz = 0;
   int buf_pf = 0, buf_pi = 0, rows_pi = 0;     // complex elements per plane buffer
@@ -405,8 +436,8 @@ struct psatd_plan {
   std::vector<void*> allocs;
   BoxDev* d_boxes = nullptr;
   ShapeDev* d_shapes = nullptr;
-  RowJob *d_rows_all = nullptr, *d_rows_int = nullptr;
-  ColJob *d_ycols_all = nullptr, *d_ycols_int = nullptr, *d_zcols = nullptr;
+  RowJob* d_rows_all = nullptr;
+  ColJob *d_ycols_all = nullptr, *d_zcols = nullptr;
   RowJob *d_g_rows = nullptr, *d_g_rows_int = nullptr;
   ColJob *d_g_ycols = nullptr, *d_g_ycols_int = nullptr, *d_g_zcols = nullptr, *d_zfast = nullptr;
   int2 *d_plane_fwd = nullptr, *d_plane_inv = nullptr;
@@ -711,7 +742,7 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
     s.L = b.n[0] / 2;
     s.hx = s.L + 1;
     s.p = b.order_p;
-    if (!radix_plan(s.L, s.ax) || !radix_plan(b.n[1], s.ay) || !radix_plan(b.n[2], s.az))
+    if (!line_plan(s.L, s.ax) || !line_plan(b.n[1], s.ay) || !line_plan(b.n[2], s.az))
       return fail(nullptr, PSATD_ERR_UNSUPPORTED_SIZE, "no radix schedule");
     s.ax.tw = tw_offset(s.L);
     s.ay.tw = tw_offset(b.n[1]);
@@ -775,7 +806,6 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
   P->spec_total = soff;
   // ---- work lists
   const int csz = (int)P->csize;
-  const int zbudget = 100 * 1024;
   int dev = 0, optin = 0;
   CK(P, cudaGetDevice(&dev));
   CK(P, cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
@@ -813,6 +843,9 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
     return P->reg_planes ? c : -1;
   };
   std::vector<int> box_reg(P->boxes.size(), -1);
+  std::vector<char> box_generic(P->boxes.size(), 0);
+  int64_t zcolumns = 0;          // z columns of the generic boxes
+  int zlongest = 0, zany = 0;    // their longest z line, and any box's
   for (int bi = 0; bi < (int)P->boxes.size(); ++bi) {
     const psatd_box& b = P->boxes[bi];
     const int n0 = b.n[0], n1 = b.n[1], n2 = b.n[2];
@@ -823,12 +856,8 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
     const int sm_zf = z_fast_smem(P->prec, P->form, n2);
     const bool fast_ok = plane_ok(b, sh);
     const int rows = n1 * n2;
-    const int nr = std::max(1, std::min(rows, kMaxPoints / L));
+    const int nr = line_tile_width(P->prec);
     for (int r = 0; r < rows; r += nr) P->rows_all.push_back({bi, r, std::min(nr, rows - r), 0});
-    for (int z = b.ng_lo[2]; z < n2 - b.ng_hi[2]; ++z) {
-      const int y0 = b.ng_lo[1], y1 = n1 - b.ng_hi[1];
-      for (int y = y0; y < y1; y += nr) P->rows_int.push_back({bi, z * n1 + y, std::min(nr, y1 - y), 0});
-    }
     const bool pencil_ok = !(d.flags & PSATD_GENERIC_KERNELS) && P->form != kPml && sh.px >= 0 && sh.py >= 0 &&
                            sh.pz >= 0 &&
                            n2 <= pen_z_max(P->prec) && sm_zf <= optin && pen_col_smem(P->prec, n1) <= optin;
@@ -837,7 +866,8 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
         (d.flags & PSATD_PENCIL_KERNELS) || (!(d.flags & PSATD_PLANE_KERNELS) && box_reg[bi] < 0);
     const bool fast = (fast_ok || box_reg[bi] >= 0) && !(pencil_ok && prefer_pencil);
     const bool pencil = !fast && pencil_ok;
-    const bool generic = !fast && !pencil;   // the generic Stockham kernels
+    const bool generic = !fast && !pencil;   // the generic kernels
+    box_generic[bi] = generic;
     if (fast) {
       ++P->fast_boxes;
       for (int z = 0; z < n2; ++z) {
@@ -891,35 +921,32 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
         for (int y = y0; y < y1; y += nr) P->g_rows_int.push_back({bi, z * n1 + y, std::min(nr, y1 - y), 0});
       }
     }
-    P->smem_fx = std::max(P->smem_fx, nr * L * csz);
-    P->smem_ix = std::max(P->smem_ix, nr * (hx + L) * csz);
-    int ny = std::max(1, kMaxPoints / n1);
-    if (ny >= 8) ny = ny / 8 * 8;
-    ny = std::min(ny, hx);
-    for (int z = 0; z < n2; ++z) {
-      const bool inner = z >= b.ng_lo[2] && z < n2 - b.ng_hi[2];
-      for (int m = 0; m < hx; m += ny) {
-        ColJob j{bi, z, m, std::min(ny, hx - m)};
-        P->ycols_all.push_back(j);
-        if (inner) P->ycols_int.push_back(j);
-        if (generic) {
-          P->g_ycols.push_back(j);
-          if (inner) P->g_ycols_int.push_back(j);
-        }
-      }
+    line_cover(P->cfg_fx, P->prec, sh.ax, 1);
+    line_cover(P->cfg_ix, P->prec, sh.ax, 2);
+    line_cover(P->cfg_y, P->prec, sh.ay, 0);
+    line_cover(P->cfg_zonly, P->prec, sh.az, 0);
+    // column tiles run on through the planes
+    const int yi0 = b.ng_lo[2], yi1 = n2 - b.ng_hi[2];
+    column_tiles(P->ycols_all, bi, 0, n2, hx, nr);
+    column_tiles(P->zcols, bi, 0, n1, hx, nr);
+    if (generic) {
+      column_tiles(P->g_ycols, bi, 0, n2, hx, nr);
+      column_tiles(P->g_ycols_int, bi, yi0, yi1, hx, nr);
+      zcolumns += (int64_t)n1 * hx;
+      zlongest = std::max(zlongest, n2);
     }
-    P->smem_y = std::max(P->smem_y, n1 * ny * csz);
-    int nz = std::max(1, zbudget / (n2 * spec_slots(P->form) * csz));
-    if (nz >= 4) nz = nz / 4 * 4;
-    nz = std::min(nz, hx);
-    for (int y = 0; y < n1; ++y)
-      for (int m = 0; m < hx; m += nz) {
-        P->zcols.push_back({bi, y, m, std::min(nz, hx - m)});
-        if (generic) P->g_zcols.push_back({bi, y, m, std::min(nz, hx - m)});
-      }
-    P->smem_z = std::max(P->smem_z, n2 * spec_slots(P->form) * nz * csz);
-    P->smem_zonly = std::max(P->smem_zonly, n2 * nz * csz);
   }
+  // the generic z pass: its tile width follows the longest line and the number of columns
+  for (const psatd_box& b : P->boxes) zany = std::max(zany, b.n[2]);
+  z_cover(P->cfg_z, P->prec, P->form, zlongest ? zlongest : zany, zlongest ? zcolumns : INT64_MAX, P->sms, optin);
+  for (const psatd_box& b : P->boxes) {
+    AxisPlan a{};
+    line_plan(b.n[2], a);
+    if (std::max(a.r1, a.r2) > 16) P->cfg_z.cls = 1;
+  }
+  for (int bi = 0; bi < (int)P->boxes.size(); ++bi)
+    if (box_generic[bi])
+      column_tiles(P->g_zcols, bi, 0, P->boxes[bi].n[1], P->boxes[bi].n[0] / 2 + 1, 1 << P->cfg_z.lg);
   // pencil jobs grouped by the FFT length of the axis each kernel transforms
   // (one launch per group; boxes keep their order inside a group)
   auto group = [&](auto& list, auto code_of, std::vector<psatd_plan::PenGroup>& groups) {
@@ -1106,9 +1133,7 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
   CK(P, upload(P, P->hboxes, &P->d_boxes));
   CK(P, upload(P, P->hshapes, &P->d_shapes));
   CK(P, upload(P, P->rows_all, &P->d_rows_all));
-  CK(P, upload(P, P->rows_int, &P->d_rows_int));
   CK(P, upload(P, P->ycols_all, &P->d_ycols_all));
-  CK(P, upload(P, P->ycols_int, &P->d_ycols_int));
   CK(P, upload(P, P->zcols, &P->d_zcols));
   CK(P, upload(P, P->g_rows, &P->d_g_rows));
   CK(P, upload(P, P->g_rows_int, &P->d_g_rows_int));
@@ -1193,7 +1218,7 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   free_tmp();
   CK(P, e);
-  const int smem = std::max({P->smem_fx, P->smem_y, P->smem_z, P->smem_zonly, P->smem_ix, P->smem_pf,
+  const int smem = std::max({P->cfg_fx.smem, P->cfg_y.smem, P->cfg_z.smem, P->cfg_zonly.smem, P->cfg_ix.smem, P->smem_pf,
                              P->smem_pi, P->smem_zf, P->smem_penx, P->smem_penxi, P->smem_penc, P->smem_penz});
   if (smem > optin) return fail(P, PSATD_ERR_UNSUPPORTED_SIZE, fmt("needs %d B shared memory", smem));
   // The attribute is a per-kernel cap shared by every plan: raise it to the
@@ -1692,10 +1717,10 @@ static psatd_status forward_xy(psatd_plan* P, const DevPlan& D, const FieldPtrs&
   }
   if (!P->g_rows.empty()) {
     CK(P, timed(P, 0, st, [&] {
-         return launch_fwd_x(P->prec, D, fp, nf, spec, S, P->d_g_rows, (int64_t)P->g_rows.size(), P->smem_fx, st);
+         return launch_fwd_x(P->prec, D, fp, nf, spec, S, P->d_g_rows, (int64_t)P->g_rows.size(), P->cfg_fx, st);
        }));
     CK(P, timed(P, 1, st, [&] {
-         return launch_col(P->prec, -1, 1, D, spec, S, nf, P->d_g_ycols, (int64_t)P->g_ycols.size(), P->smem_y, st);
+         return launch_col(P->prec, -1, 1, D, spec, S, nf, P->d_g_ycols, (int64_t)P->g_ycols.size(), P->cfg_y, st);
        }));
     launches += 2;
   }
@@ -1761,7 +1786,7 @@ static psatd_status transform_current(psatd_plan* P, const DevPlan& D, const Fie
   }
   CK(P, timed(P, 2, st, [&] {
        return launch_col(P->prec, -1, 2, D, spec, P->spec_total, 3, P->d_zcols, (int64_t)P->zcols.size(),
-                         P->smem_zonly, st);
+                         P->cfg_zonly, st);
      }));
   ++*launches_out;
   return PSATD_OK;
@@ -1811,7 +1836,7 @@ static psatd_status z_step(psatd_plan* P, const DevPlan& D, cudaStream_t st, int
   }
   if (!P->g_zcols.empty()) {
     CK(P, timed(P, 2, st, [&] {
-         return launch_z_update(P->prec, P->form, D, P->d_ws, S, P->d_g_zcols, (int64_t)P->g_zcols.size(), P->smem_z,
+         return launch_z_update(P->prec, P->form, D, P->d_ws, S, P->d_g_zcols, (int64_t)P->g_zcols.size(), P->cfg_z,
                                 NFT, st);
        }));
     ++launches;
@@ -1859,10 +1884,10 @@ static psatd_status inverse_step(psatd_plan* P, const DevPlan& D, const FieldPtr
   }
   if (!P->g_rows.empty()) {
     CK(P, timed(P, 3, st, [&] {
-         return launch_col(P->prec, 1, 1, D, spec, S, nout, P->d_g_ycols_int, (int64_t)P->g_ycols_int.size(), P->smem_y, st);
+         return launch_col(P->prec, 1, 1, D, spec, S, nout, P->d_g_ycols_int, (int64_t)P->g_ycols_int.size(), P->cfg_y, st);
        }));
     CK(P, timed(P, 4, st, [&] {
-         return launch_inv_x(P->prec, D, fp, nout, spec, S, P->d_g_rows_int, (int64_t)P->g_rows_int.size(), P->smem_ix, 1, st);
+         return launch_inv_x(P->prec, D, fp, nout, spec, S, P->d_g_rows_int, (int64_t)P->g_rows_int.size(), P->cfg_ix, 1, st);
        }));
     launches += 2;
   }
@@ -2224,9 +2249,9 @@ psatd_status psatd_forward_fft(psatd_plan* P, const void* field, void* spectrum,
   P->last_stream = st;
   const DevPlan D = P->dev();
   const int64_t S = P->spec_total;
-  CK(P, launch_fwd_x(P->prec, D, fp, 1, spectrum, S, P->d_rows_all, (int64_t)P->rows_all.size(), P->smem_fx, st));
-  CK(P, launch_col(P->prec, -1, 1, D, spectrum, S, 1, P->d_ycols_all, (int64_t)P->ycols_all.size(), P->smem_y, st));
-  CK(P, launch_col(P->prec, -1, 2, D, spectrum, S, 1, P->d_zcols, (int64_t)P->zcols.size(), P->smem_zonly, st));
+  CK(P, launch_fwd_x(P->prec, D, fp, 1, spectrum, S, P->d_rows_all, (int64_t)P->rows_all.size(), P->cfg_fx, st));
+  CK(P, launch_col(P->prec, -1, 1, D, spectrum, S, 1, P->d_ycols_all, (int64_t)P->ycols_all.size(), P->cfg_y, st));
+  CK(P, launch_col(P->prec, -1, 2, D, spectrum, S, 1, P->d_zcols, (int64_t)P->zcols.size(), P->cfg_zonly, st));
   P->last_launches = 3;
   return PSATD_OK;
 }
@@ -2241,9 +2266,9 @@ psatd_status psatd_inverse_fft(psatd_plan* P, void* spectrum, void* field, void*
   P->last_stream = st;
   const DevPlan D = P->dev();
   const int64_t S = P->spec_total;
-  CK(P, launch_col(P->prec, 1, 2, D, spectrum, S, 1, P->d_zcols, (int64_t)P->zcols.size(), P->smem_zonly, st));
-  CK(P, launch_col(P->prec, 1, 1, D, spectrum, S, 1, P->d_ycols_all, (int64_t)P->ycols_all.size(), P->smem_y, st));
-  CK(P, launch_inv_x(P->prec, D, fp, 1, spectrum, S, P->d_rows_all, (int64_t)P->rows_all.size(), P->smem_ix, 0, st));
+  CK(P, launch_col(P->prec, 1, 2, D, spectrum, S, 1, P->d_zcols, (int64_t)P->zcols.size(), P->cfg_zonly, st));
+  CK(P, launch_col(P->prec, 1, 1, D, spectrum, S, 1, P->d_ycols_all, (int64_t)P->ycols_all.size(), P->cfg_y, st));
+  CK(P, launch_inv_x(P->prec, D, fp, 1, spectrum, S, P->d_rows_all, (int64_t)P->rows_all.size(), P->cfg_ix, 0, st));
   P->last_launches = 3;
   return PSATD_OK;
 }
@@ -2293,25 +2318,13 @@ psatd_status psatd_plan_distribute(psatd_plan* P, int32_t world, int32_t rank) {
     const int ib = (int)hb.size();
     hb.push_back(slab);
     hb.push_back(rows);
-    // the tile sizes of the plan's generic kernels (its shared-memory limits hold)
-    const int csz = (int)P->csize;
+    // the tile sizes of the plan's generic kernels (the same lengths, so its launches cover them)
     std::vector<RowJob> rj;
-    const int nr = std::max(1, std::min(nz * n1, kMaxPoints / L));
+    const int nr = line_tile_width(P->prec);
     for (int r = 0; r < nz * n1; r += nr) rj.push_back({ib, r, std::min(nr, nz * n1 - r), 0});
     std::vector<ColJob> yc, zc;
-    int tyc = std::max(1, kMaxPoints / n1);
-    if (tyc >= 8) tyc = tyc / 8 * 8;
-    tyc = std::min(tyc, hx);
-    for (int z = 0; z < nz; ++z)
-      for (int m = 0; m < hx; m += tyc) yc.push_back({ib, z, m, std::min(tyc, hx - m)});
-    int tzc = std::max(1, 100 * 1024 / (n2 * spec_slots(P->form) * csz));
-    if (tzc >= 4) tzc = tzc / 4 * 4;
-    tzc = std::min(tzc, hx);
-    for (int y = 0; y < ny; ++y)
-      for (int m = 0; m < hx; m += tzc) zc.push_back({ib + 1, y, m, std::min(tzc, hx - m)});
-    if (nr * L * csz > P->smem_fx || nr * (hx + L) * csz > P->smem_ix || n1 * tyc * csz > P->smem_y ||
-        n2 * spec_slots(P->form) * tzc * csz > P->smem_z)
-      return fail(P, PSATD_ERR_UNSUPPORTED_SIZE, "slab tiles exceed the plan's shared memory");
+    column_tiles(yc, ib, 0, nz, hx, nr);
+    column_tiles(zc, ib + 1, 0, ny, hx, 1 << P->cfg_z.lg);
     CK(P, upload(P, hb, &d.d_boxes));
     CK(P, upload(P, rj, &d.d_rows));
     CK(P, upload(P, yc, &d.d_ycols));
@@ -2351,8 +2364,8 @@ psatd_status psatd_dist_forward_xy(psatd_plan* P, const psatd_fields* slab, cons
   DevPlan D = P->dev();
   D.boxes = P->dist.d_boxes;
   const auto& d = P->dist;
-  CK(P, launch_fwd_x(P->prec, D, fp, nf, slab_spectrum, d.s_slab, d.d_rows, d.nrows, P->smem_fx, st));
-  CK(P, launch_col(P->prec, -1, 1, D, slab_spectrum, d.s_slab, nf, d.d_ycols, d.nycols, P->smem_y, st));
+  CK(P, launch_fwd_x(P->prec, D, fp, nf, slab_spectrum, d.s_slab, d.d_rows, d.nrows, P->cfg_fx, st));
+  CK(P, launch_col(P->prec, -1, 1, D, slab_spectrum, d.s_slab, nf, d.d_ycols, d.nycols, P->cfg_y, st));
   P->last_launches = 2;
   return PSATD_OK;
 }
@@ -2366,7 +2379,7 @@ psatd_status psatd_dist_z_update(psatd_plan* P, void* rows, void* stream) {
   DevPlan D = P->dev();
   D.boxes = P->dist.d_boxes;
   const auto& d = P->dist;
-  CK(P, launch_z_update(P->prec, P->form, D, rows, d.s_rows, d.d_zcols, d.nzcols, P->smem_z, fields_in(P->form),
+  CK(P, launch_z_update(P->prec, P->form, D, rows, d.s_rows, d.d_zcols, d.nzcols, P->cfg_z, fields_in(P->form),
                         st));
   P->last_launches = 1;
   return PSATD_OK;
@@ -2388,8 +2401,8 @@ psatd_status psatd_dist_inverse_yx(psatd_plan* P, void* slab_spectrum, const psa
   DevPlan D = P->dev();
   D.boxes = P->dist.d_boxes;
   const auto& d = P->dist;
-  CK(P, launch_col(P->prec, 1, 1, D, slab_spectrum, d.s_slab, FOUT, d.d_ycols, d.nycols, P->smem_y, st));
-  CK(P, launch_inv_x(P->prec, D, fp, FOUT, slab_spectrum, d.s_slab, d.d_rows, d.nrows, P->smem_ix, 1, st));
+  CK(P, launch_col(P->prec, 1, 1, D, slab_spectrum, d.s_slab, FOUT, d.d_ycols, d.nycols, P->cfg_y, st));
+  CK(P, launch_inv_x(P->prec, D, fp, FOUT, slab_spectrum, d.s_slab, d.d_rows, d.nrows, P->cfg_ix, 1, st));
   P->last_launches = 2;
   return PSATD_OK;
 }

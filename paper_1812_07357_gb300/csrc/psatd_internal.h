@@ -11,10 +11,7 @@
 
 namespace psatd {
 
-constexpr int kMaxPass = 16;       // radix passes of one axis (2^10 needs <= 4 with radix 8)
-constexpr int kThreads = 256;      // threads per CTA of every FFT kernel
-constexpr int kPointsPerThread = 16;
-constexpr int kMaxPoints = kThreads * kPointsPerThread;  // points of one FFT chunk in smem
+constexpr int kThreads = 256;      // threads per CTA of the plane and pencil z kernels
 
 // Equation form of the k-space update (slot layout of the fields):
 //   kVacuum: E 0-2, B 3-5                      (6 in, 6 out)
@@ -30,12 +27,22 @@ constexpr int fields_out(int form) { return form == kRhoForm ? 7 : form == kPml 
 // spectrum slots a step needs (inputs and outputs share them)
 constexpr int spec_slots(int form) { return fields_in(form) > fields_out(form) ? fields_in(form) : fields_out(form); }
 
-// Radix schedule of one complex FFT length.
+// One complex FFT length n = r1 * r2 and its index maps (any_fft.cuh).
 struct AxisPlan {
   int32_t n;
-  int32_t npass;
+  int32_t r1, r2;
+  int32_t wrap;                   // 1: prime-factor maps (no twiddles), 0: decimation in time
+  int32_t a_in;                   // first sample of sub-transform n2: a_in * n2; then every r2-th (mod n)
+  int32_t a_out, s_out;           // output (k1, k2): (a_out k1 + s_out k2) mod n
+  int32_t pad;
   int64_t tw;                     // offset of the n-entry twiddle table (complex pool)
-  uint8_t radix[kMaxPass];
+};
+
+// Launch of a generic kernel over lines of several lengths: the largest shared
+// memory and block any of them needs, the class of the largest radix, and the
+// logarithm of the z pass's tile width.
+struct LineCfg {
+  int smem = 0, threads = 0, cls = 0, lg = 0;
 };
 
 // Tables of one box shape (n0, n1, n2, p); offsets index the typed pools.
@@ -102,7 +109,8 @@ struct RowJob {
 
 // columns m0 .. m0+nm-1 of one plane (y-axis passes: plane = z; z-axis: plane = y).
 // Fast z tiles with nm < 0 hold the Nyquist column mx = m0 = n0/2 of the -nm
-// planes y = plane .. plane-nm-1.
+// planes y = plane .. plane-nm-1.  Tiles of the generic kernels run on from
+// column n0/2 of a plane to column 0 of the next.
 struct ColJob {
   int32_t box, plane, m0, nm;
 };
@@ -181,24 +189,30 @@ inline void set_constants(DevPlan& P, double c, double eps0, double dt) {
   P.icce = 1.0 / (c * c * eps0);
 }
 
-// ---- kernel launchers (fft_kernels.cu, exchange.cu) ----------------------
+// ---- generic kernels (fft_kernels.cu, any_z.cu) ---------------------------
 
-// Forward R2C along x of `nf` field slots into spectrum slots (stride sstride).
-cudaError_t launch_fwd_x(int prec, const DevPlan& P, const FieldPtrs& f, int nf, void* spec,
-                         int64_t sstride, const RowJob* jobs, int64_t njobs, int smem,
-                         cudaStream_t st);
-// Complex FFT along y (axis 1) or z (axis 2), in place on spectrum slots.
-cudaError_t launch_col(int prec, int dir, int axis, const DevPlan& P, void* spec,
-                       int64_t sstride, int nf, const ColJob* jobs, int64_t njobs, int smem,
-                       cudaStream_t st);
-// z forward FFT + k-space update + z inverse FFT, all slots of `form`.
+// Forward R2C along x of `nf` field slots into spectrum slots (stride
+// sstride); row jobs of at most line_tile_width rows.
+cudaError_t launch_fwd_x(int prec, const DevPlan& P, const FieldPtrs& f, int nf, void* spec, int64_t sstride,
+                         const RowJob* jobs, int64_t njobs, const LineCfg& c, cudaStream_t st);
+// Complex FFT along y (axis 1) or z (axis 2), in place on spectrum slots;
+// column jobs of at most line_tile_width columns.
+cudaError_t launch_col(int prec, int dir, int axis, const DevPlan& P, void* spec, int64_t sstride, int nf,
+                       const ColJob* jobs, int64_t njobs, const LineCfg& c, cudaStream_t st);
+// z forward FFT + k-space update + z inverse FFT, all slots of `form`; jobs of
+// at most 2^c.lg columns.
 // nft: field slots transformed along z (the others hold a cached z spectrum)
-cudaError_t launch_z_update(int prec, int form, const DevPlan& P, void* spec, int64_t sstride,
-                            const ColJob* jobs, int64_t njobs, int smem, int nft, cudaStream_t st);
+cudaError_t launch_z_update(int prec, int form, const DevPlan& P, void* spec, int64_t sstride, const ColJob* jobs,
+                            int64_t njobs, const LineCfg& c, int nft, cudaStream_t st);
 // C2R inverse along x with 1/(n0 n1 n2) into field slots; interior_only skips guards.
-cudaError_t launch_inv_x(int prec, const DevPlan& P, const FieldPtrs& f, int nf, void* spec,
-                         int64_t sstride, const RowJob* jobs, int64_t njobs, int smem,
-                         int interior_only, cudaStream_t st);
+cudaError_t launch_inv_x(int prec, const DevPlan& P, const FieldPtrs& f, int nf, void* spec, int64_t sstride,
+                         const RowJob* jobs, int64_t njobs, const LineCfg& c, int interior_only, cudaStream_t st);
+int line_tile_width(int prec);   // rows or columns of a tile
+void line_cover(LineCfg& c, int prec, const AxisPlan& a, int kind);
+void z_cover(LineCfg& c, int prec, int form, int n2_max, int64_t columns, int sms, int optin);
+cudaError_t configure_any_z(int prec, int smem_bytes);
+
+// ---- exchange (exchange.cu) -------------------------------------------------
 // Guard exchange of `nf` field slots.
 // Absorbing layers, step (2): one box of the layers' list.  Damping table
 // (type T): for axis d and Yee offset o (0: cell, 1: half cell), entry
@@ -326,8 +340,12 @@ cudaError_t launch_pen_xi(int prec, int code, const DevPlan& P, const FieldPtrs&
 cudaError_t configure_pen_kernels(int prec, int smem_bytes);
 
 // ---- host helpers (plan.cpp) ------------------------------------------------
-// Radix schedule of a complex FFT length (false if it is not 5-smooth).
-bool radix_plan(int n, AxisPlan& ap);
+// Two radices and the index maps of a complex FFT length (false when there are
+// none: not 5-smooth, or above 1024).
+bool line_plan(int n, AxisPlan& ap);
+// Tiles of `w` columns of the planes [p0, p1) of a box, hx columns each, the
+// columns numbered through the planes.
+void column_tiles(std::vector<ColJob>& out, int box, int p0, int p1, int hx, int w);
 // Weights alpha_l, l = 1..p/2, of the order-p staggered difference
 // (nodal: beta_l of the centred collocated difference).
 std::vector<double> stencil_alpha(int p, bool nodal = false);

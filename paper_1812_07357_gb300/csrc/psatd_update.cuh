@@ -353,6 +353,30 @@ __device__ __forceinline__ void update_core2(C2* m, float2 Kx, float2 Ky, float2
     ney = eg(ney, x1y);
     nez = eg(nez, x1z);
   }
+  if constexpr (FORM == kPml) {
+    // increments of the stored split parts (see update_core)
+    const C2 kde = dot3(Kx, ex, Ky, ey, Kz, ez);
+    const float2 X1 = q.x1, nX1 = neg2(q.x1), nX3 = neg2(q.x3);
+    const float2 x1c = mul2(q.x1, bcast<float2>(P.icce * P.eps0)), nx1c = neg2(x1c);
+    // I[E] = S E - X3 K (K.E) + i X1 K x B,  I[B] = S B - X3 K (K.B) - i (X1/c^2) K x E
+    auto inc = [&](C2 f, float2 k, C2 kdf, float2 w, float2 nw, C2 kx) {
+      const float2 a = mul2(nX3, k);
+      return C2{fma2(nw, kx.y, fma2(a, kdf.x, mul2(S, f.x))), fma2(w, kx.x, fma2(a, kdf.y, mul2(S, f.y)))};
+    };
+    const C2 iex = inc(ex, Kx, kde, X1, nX1, kbx), iey = inc(ey, Ky, kde, X1, nX1, kby),
+             iez = inc(ez, Kz, kde, X1, nX1, kbz);
+    const C2 ibx = inc(bx, Kx, kdb, nx1c, x1c, kex), iby = inc(by, Ky, kdb, nx1c, x1c, key),
+             ibz = inc(bz, Kz, kdb, nx1c, x1c, kez);
+    // i w a for real w, given as (w, -w)
+    auto itimes = [&](float2 w, float2 nw, C2 a) { return C2{mul2(nw, a.y), mul2(w, a.x)}; };
+    const float2 ckx = mul2(cc, Kx), cky = mul2(cc, Ky), ckz = mul2(cc, Kz);
+    m[6] = cmul_n(itimes(cky, neg2(cky), ibz), px, npx);
+    m[7] = cmul_n(itimes(ckz, neg2(ckz), ibx), py, npy);
+    m[8] = cmul_n(itimes(ckx, neg2(ckx), iby), pz, npz);
+    m[9] = cmul_n(itimes(nKy, Ky, iez), pyz, npyz);
+    m[10] = cmul_n(itimes(nKz, Kz, iex), pxz, npxz);
+    m[11] = cmul_n(itimes(nKx, Kx, iey), pxy, npxy);
+  }
   // back to the staggered sample positions
   m[0] = cmul_n(nex, px, npx);
   m[1] = cmul_n(ney, py, npy);
@@ -405,12 +429,6 @@ __device__ __forceinline__ void update_pair_z2(float2* lo, float2* hi, int fs, c
     store2<false>(lo + f * fs, a[f] + b[f]);
     store2<true>(hi + f * fs, cmulc(a[f] - b[f], W));
   }
-}
-
-template <typename T, int FORM>
-__device__ __forceinline__ void update_mode(cx<T>* md, int fs, int mx, int my, int mz,
-                                            const ShapeDev& sh, const DevPlan& P) {
-  update_mode_z<T, FORM>(md, fs, mode_xy<T>(mx, my, sh, P), mz, sh, P);
 }
 
 }  // namespace psatd

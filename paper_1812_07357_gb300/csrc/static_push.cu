@@ -107,7 +107,7 @@ extern "C" psatd_status psatd_push_box_static(const int32_t n[3], int32_t order_
   s.L = L;
   s.hx = hx;
   s.p = order_p;
-  if (!radix_plan(L, s.ax) || !radix_plan(n1, s.ay) || !radix_plan(n2, s.az))
+  if (!line_plan(L, s.ax) || !line_plan(n1, s.ay) || !line_plan(n2, s.az))
     return err(PSATD_ERR_UNSUPPORTED_SIZE, "no radix schedule");
   int64_t ctot = 0, rtot = 0;
   auto ctake = [&](int64_t k) {
@@ -137,19 +137,18 @@ extern "C" psatd_status psatd_push_box_static(const int32_t n[3], int32_t order_
   const int64_t spec = (int64_t)hx * n1 * n2;
   std::vector<RowJob> rows;
   std::vector<ColJob> ycols, zcols;
-  const int nr = std::max(1, std::min(n1 * n2, kMaxPoints / L));
+  const int nr = line_tile_width(32);
   for (int r = 0; r < n1 * n2; r += nr) rows.push_back({0, r, std::min(nr, n1 * n2 - r), 0});
-  int ny = std::max(1, kMaxPoints / n1);
-  if (ny >= 8) ny = ny / 8 * 8;
-  ny = std::min(ny, hx);
-  for (int z = 0; z < n2; ++z)
-    for (int m = 0; m < hx; m += ny) ycols.push_back({0, z, m, std::min(ny, hx - m)});
-  int nz = std::max(1, 100 * 1024 / (n2 * FIN * 8));
-  if (nz >= 4) nz = nz / 4 * 4;
-  nz = std::min(nz, hx);
-  for (int y = 0; y < n1; ++y)
-    for (int m = 0; m < hx; m += nz) zcols.push_back({0, y, m, std::min(nz, hx - m)});
-  const int smem = std::max({nr * L * 8, n1 * ny * 8, n2 * FIN * nz * 8, nr * (hx + L) * 8});
+  column_tiles(ycols, 0, 0, n2, hx, nr);
+  LineCfg cfx, cix, cy, cz;
+  line_cover(cfx, 32, s.ax, 1);
+  line_cover(cix, 32, s.ax, 2);
+  line_cover(cy, 32, s.ay, 0);
+  // two tiles per SM of the largest part, so that the lists do not depend on the device
+  z_cover(cz, 32, kVacuum, n2, (int64_t)n1 * hx, 160, 200 * 1024);
+  cz.cls = std::max(s.az.r1, s.az.r2) > 16;
+  column_tiles(zcols, 0, 0, n1, hx, 1 << cz.lg);
+  const int smem = std::max({cfx.smem, cix.smem, cy.smem, cz.smem});
   const std::vector<double> alpha = order_p ? stencil_alpha(order_p) : std::vector<double>(1, 0.0);
 
   // ---- carve the arena: [box][shape][rows][ycols][zcols][alpha][r32][c32][q32][r64][c64][q64][spectra]
@@ -252,11 +251,11 @@ extern "C" psatd_status psatd_push_box_static(const int32_t n[3], int32_t order_
   const ColJob* dy = reinterpret_cast<const ColJob*>(A + o_ycols);
   const ColJob* dz = reinterpret_cast<const ColJob*>(A + o_zcols);
   for (int step = 0; step < nsteps; ++step) {
-    PSATD_CK(launch_fwd_x(32, P, fp, FIN, ws, spec, drows, (int64_t)rows.size(), nr * L * 8, st));
-    PSATD_CK(launch_col(32, -1, 1, P, ws, spec, FIN, dy, (int64_t)ycols.size(), n1 * ny * 8, st));
-    PSATD_CK(launch_z_update(32, kVacuum, P, ws, spec, dz, (int64_t)zcols.size(), n2 * FIN * nz * 8, FIN, st));
-    PSATD_CK(launch_col(32, 1, 1, P, ws, spec, FIN, dy, (int64_t)ycols.size(), n1 * ny * 8, st));
-    PSATD_CK(launch_inv_x(32, P, fp, FIN, ws, spec, drows, (int64_t)rows.size(), nr * (hx + L) * 8, 1, st));
+    PSATD_CK(launch_fwd_x(32, P, fp, FIN, ws, spec, drows, (int64_t)rows.size(), cfx, st));
+    PSATD_CK(launch_col(32, -1, 1, P, ws, spec, FIN, dy, (int64_t)ycols.size(), cy, st));
+    PSATD_CK(launch_z_update(32, kVacuum, P, ws, spec, dz, (int64_t)zcols.size(), cz, FIN, st));
+    PSATD_CK(launch_col(32, 1, 1, P, ws, spec, FIN, dy, (int64_t)ycols.size(), cy, st));
+    PSATD_CK(launch_inv_x(32, P, fp, FIN, ws, spec, drows, (int64_t)rows.size(), cix, 1, st));
   }
 #undef PSATD_CK
   return PSATD_OK;
