@@ -19,8 +19,9 @@ LIBDIR = os.path.join(PKG, "lib")
 LIB = os.path.join(LIBDIR, "libpsatd.so")
 BUILD = os.path.join(PKG, "_build")
 
-SOURCES = ["plan.cpp", "tables.cu", "fft_kernels.cu", "any_z.cu", "fast_kernels.cu", "reg_kernels.cu", "reg_planes_0.cu",
-           "reg_planes_1.cu", "reg_planes_2.cu", "reg_planes_3.cu", "pencil_kernels.cu", "exchange.cu", "static_push.cu"]
+SOURCES = ["plan.cpp", "tables.cu", "fft_kernels.cu", "any_part_0.cu", "any_part_1.cu",
+           "any_part_2.cu", "any_part_3.cu", "fast_kernels.cu", "reg_kernels.cu", "reg_planes_0.cu",
+           "reg_planes_1.cu", "reg_planes_2.cu", "reg_planes_3.cu", "exchange.cu", "static_push.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -1,5 +1,5 @@
 // FFT lines of any 5-smooth length up to 512, the building block of the
-// generic kernels (fft_kernels.cu, any_z.cu): every length is done in two
+// generic kernels (any_lines.cuh, any_z.cuh): every length is done in two
 // register passes over run-time radices,
 //
 //   N = r1 * r2:  pass 1, one thread per (line, n2): a DFT of the r1 samples
@@ -38,6 +38,19 @@ namespace {
 template <typename T>
 __host__ __device__ constexpr int line_tile() {
   return 128 / (2 * (int)sizeof(T));
+}
+
+// Row pitch of the FP32 x kernels in shared memory: sub-transform k1 at
+// k1 * (r2 | 1), so that lanes along n2 and lanes along k1 both read it without
+// bank conflicts; the natural-order row needs r1 * r2 of it.
+__host__ __device__ __forceinline__ int row_line_pitch(const AxisPlan& a) { return a.r1 * (a.r2 | 1); }
+
+// complex elements between two slots of a z tile: n2 * tx and a pad that makes
+// the pitch half a 128-byte line (mod 128 bytes)
+__host__ __device__ constexpr int z_slot_pitch(int csz, int n2, int tx) {
+  const int half = 64 / csz, line = 128 / csz;
+  const int p = n2 * tx;
+  return p + (half + line - p % line) % line;
 }
 
 // Threads of a block at most: a tile times the largest radix of the class
@@ -108,19 +121,20 @@ struct Line {
 
 // Pass 1 of sub-transform n2: load(i) gives sample i, store(k1, i, v) takes
 // result k1, whose place in an in-place transform is sample index i.
-template <typename T, int R, int DIR, typename Load, typename Store>
+// WRAP = false: a length planned without prime-factor maps.
+template <typename T, int R, int DIR, bool WRAP, typename Load, typename Store>
 __device__ __forceinline__ void line_pass1(const Line& l, int n2, const cx<T>* __restrict__ tw, Load&& load,
                                            Store&& store) {
   cx<T> v[R];
-  const int i0 = l.a_in * n2;
+  const int i0 = WRAP ? l.a_in * n2 : n2;
   int i = i0;
 #pragma unroll
   for (int j = 0; j < R; ++j) {
     v[j] = load(i);
-    i = l.next(i, l.r2);
+    i = WRAP ? l.next(i, l.r2) : i + l.r2;
   }
   Dft<T, R, DIR>::run(v);
-  if (!l.wrap && n2) {
+  if (!(WRAP && l.wrap) && n2) {
 #pragma unroll
     for (int k = 1; k < R; ++k) v[k] = twmul<DIR>(v[k], tw[n2 * k]);
   }
@@ -128,7 +142,7 @@ __device__ __forceinline__ void line_pass1(const Line& l, int n2, const cx<T>* _
 #pragma unroll
   for (int k = 0; k < R; ++k) {
     store(k, i, v[k]);
-    i = l.next(i, l.r2);
+    i = WRAP ? l.next(i, l.r2) : i + l.r2;
   }
 }
 

@@ -13,6 +13,8 @@
 // [slot][place][column], the slots half a 128-byte line apart, so that lanes
 // over (column, place) and lanes over (column, slot) both read it without
 // bank conflicts.
+#pragma once
+
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -29,14 +31,6 @@ namespace {
 template <typename T>
 constexpr int z_threads() {   // FP64: fewer, larger threads; its pipe needs few warps
   return sizeof(T) == 4 ? 256 : 128;
-}
-
-// complex elements between two slots of a tile: n2 * tx and a pad that makes
-// the pitch half a 128-byte line (mod 128 bytes)
-__host__ __device__ constexpr int z_slot_pitch(int csz, int n2, int tx) {
-  const int half = 64 / csz, line = 128 / csz;
-  const int p = n2 * tx;
-  return p + (half + line - p % line) % line;
 }
 
 template <typename T, int FORM, int CLS>
@@ -65,7 +59,7 @@ __global__ void __launch_bounds__(z_threads<T>(), CLS ? 1 : sizeof(T) == 4 ? 2 :
         const int s = line_div(it, mr), n2i = it - s * l.r2;
         const cx<T>* gs = g + s * sstride + c;
         cx<T>* b = sm + s * SP + c;
-        line_pass1<T, decltype(rc)::value, -1>(
+        line_pass1<T, decltype(rc)::value, -1, true>(
             l, n2i, tw, [&](int i) { return gs[(int64_t)i * zst]; },
             [&](int k, int, cx<T> v) { b[(k * l.r2 + n2i) << lg] = v; });
       }
@@ -189,68 +183,5 @@ __global__ void __launch_bounds__(z_threads<T>(), CLS ? 1 : sizeof(T) == 4 ? 2 :
   }
 }
 
-template <typename T>
-cudaError_t launch_t(int form, const DevPlan& P, cx<T>* spec, int64_t sstride, const ColJob* jobs, int64_t njobs,
-                     const LineCfg& c, int nft, cudaStream_t st) {
-  const dim3 grid((unsigned)njobs);
-#define PSATD_GO(FORM)                                                                                          \
-  if (c.cls)                                                                                                    \
-    k_z_update<T, FORM, 1><<<grid, z_threads<T>(), c.smem, st>>>(P, spec, sstride, jobs, nft, c.lg);            \
-  else                                                                                                          \
-    k_z_update<T, FORM, 0><<<grid, z_threads<T>(), c.smem, st>>>(P, spec, sstride, jobs, nft, c.lg);            \
-  break
-  switch (form) {
-    case kVacuum: PSATD_GO(kVacuum);
-    case kJForm: PSATD_GO(kJForm);
-    case kPml: PSATD_GO(kPml);
-    default: PSATD_GO(kRhoForm);
-  }
-#undef PSATD_GO
-  return cudaGetLastError();
-}
-
-template <typename T, int CLS>
-cudaError_t configure_t(int smem) {
-  cudaError_t e = cudaSuccess;
-  for (const void* k : {(const void*)k_z_update<T, kVacuum, CLS>, (const void*)k_z_update<T, kJForm, CLS>,
-                        (const void*)k_z_update<T, kRhoForm, CLS>, (const void*)k_z_update<T, kPml, CLS>}) {
-    const cudaError_t r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (r != cudaSuccess) e = r;
-  }
-  return e;
-}
-
 }  // namespace
-
-cudaError_t launch_z_update(int prec, int form, const DevPlan& P, void* spec, int64_t sstride, const ColJob* jobs,
-                            int64_t njobs, const LineCfg& c, int nft, cudaStream_t st) {
-  if (njobs <= 0) return cudaSuccess;
-  if (njobs > 2147483647LL) return cudaErrorInvalidConfiguration;
-  return prec == 32 ? launch_t<float>(form, P, (float2*)spec, sstride, jobs, njobs, c, nft, st)
-                    : launch_t<double>(form, P, (double2*)spec, sstride, jobs, njobs, c, nft, st);
-}
-
-cudaError_t configure_any_z(int prec, int smem) {
-  cudaError_t e = cudaSuccess;
-  for (const cudaError_t r : {prec == 32 ? configure_t<float, 0>(smem) : configure_t<double, 0>(smem),
-                              prec == 32 ? configure_t<float, 1>(smem) : configure_t<double, 1>(smem)})
-    if (r != cudaSuccess) e = r;
-  return e;
-}
-
-// Columns per z tile (a power of two, its logarithm in c.lg) and the shared
-// memory of the longest line n2_max: the widest tile of at most 128-byte rows
-// that leaves room for three blocks per SM and gives the `columns` columns of
-// the launch at least two tiles per SM.
-void z_cover(LineCfg& c, int prec, int form, int n2_max, int64_t columns, int sms, int optin) {
-  const int csz = prec == 32 ? 8 : 16, ns = spec_slots(form);
-  const int lo = prec == 32 ? 2 : 1, hi = prec == 32 ? 4 : 3;   // log2 of the narrowest and widest tile
-  auto bytes = [&](int lg) { return ns * z_slot_pitch(csz, n2_max, 1 << lg) * csz; };
-  int lg = hi;
-  while (lg > lo && (bytes(lg) > 75 * 1024 || (columns >> lg) < 2 * sms)) --lg;
-  while (lg > 1 && bytes(lg) > optin) --lg;
-  c.lg = lg;
-  c.smem = bytes(lg);
-}
-
 }  // namespace psatd

@@ -268,10 +268,11 @@ namespace psatd {
 // Split n = r1 * r2 over the radices of the generic kernels: fewest operations
 // per point -- those of the two small DFTs (counted from the codelets: complex
 // sums, products and fused multiply-adds) and 4 per twiddle, of which coprime
-// radices need none (prime-factor maps) -- plus half an operation per unit of
-// imbalance, since the smaller radix leaves that many lanes without work.
+// radices need none (prime-factor maps) -- plus an operation per unit of
+// imbalance in FP32, half in FP64 (whose operations cost more), since the
+// smaller radix leaves that many lanes without work.
 // Radices above 16 cost registers and are taken where nothing else divides n.
-bool line_plan(int n, AxisPlan& ap) {
+bool line_plan(int n, AxisPlan& ap, int prec, bool row) {
   static const struct {
     int r;
     double ops;
@@ -297,9 +298,9 @@ bool line_plan(int n, AxisPlan& ap) {
     for (const auto& b : kRadix) {
       if (a.r * b.r != n) continue;
       const int lo = std::min(a.r, b.r), hi = std::max(a.r, b.r);
-      const bool coprime = gcd(a.r, b.r) == 1;
-      const double cost = a.ops + b.ops + (coprime ? 0.0 : 4.0 * (a.r - 1) * (b.r - 1) / n) + 0.5 * hi / lo +
-                          (hi > 16 ? 100.0 : 0.0);
+      const bool coprime = gcd(a.r, b.r) == 1 && !(row && prec == 32);
+      const double cost = a.ops + b.ops + (coprime ? 0.0 : 4.0 * (a.r - 1) * (b.r - 1) / n) +
+                          (prec == 32 ? 1.0 : 0.5) * hi / lo + (hi > 16 ? 100.0 : 0.0);
       if (cost >= best) continue;
       best = cost;
       ap = AxisPlan{};
@@ -360,23 +361,22 @@ struct psatd_plan {
 
   std::vector<BoxDev> hboxes;
   std::vector<ShapeDev> hshapes;
-  std::vector<RowJob> rows_all;
-  std::vector<ColJob> ycols_all, zcols;                      // every box (standalone FFTs)
-  std::vector<RowJob> g_rows, g_rows_int;                     // push, generic boxes
-  std::vector<ColJob> g_ycols, g_ycols_int, g_zcols;
+  // every box (standalone FFTs), the generic and pencil boxes first: those are
+  // the first g_nrows and g_nycols jobs, the x and y passes of their push
+  std::vector<RowJob> rows_all, g_rows_int;
+  std::vector<ColJob> ycols_all, zcols, g_ycols_int;
+  int64_t g_nrows = 0, g_nycols = 0;
+  std::vector<ColJob> g_zcols;                                // push, boxes on the generic z pass
   std::vector<int2> plane_fwd, plane_inv;                     // push, fast boxes
   std::vector<ColJob> zfast;
   int fast_boxes = 0;
-  std::vector<RowJob> pen_rows, pen_rows_int;                 // push, pencil boxes
-  std::vector<ColJob> pen_ycols, pen_ycols_int, zpen;
-  struct PenGroup {
-    int code;                 // pencil-length code of the transformed axis
+  struct Group {
+    int code;                 // what the group's boxes share
     int64_t start, count;     // jobs of the list
   };
-  std::vector<PenGroup> grp_rows, grp_rows_int, grp_ycols, grp_ycols_int, grp_z;
   std::vector<ColJob> zpen_reg;              // boxes of several z lengths whose z pass runs on the register z kernel
-  std::vector<PenGroup> grp_zreg;            // ... grouped by z length (code = n2)
-  std::vector<PenGroup> grp_pf, grp_pi;      // register plane jobs grouped by plane shape (code: reg_shape_code)
+  std::vector<Group> grp_zreg;               // ... grouped by z length (code = n2)
+  std::vector<Group> grp_pf, grp_pi;         // register plane jobs grouped by plane shape (code: reg_shape_code)
   // one group spread over ranks (psatd_plan_distribute): the rank's z slab
   // [z0, z1) and spectrum rows [y0, y1), the plan's boxes followed by the slab
   // box (every y, the slab's planes, the global n2 for the 1/N factor) and the
@@ -410,16 +410,14 @@ struct psatd_plan {
 
   int64_t field_total = 0;  // elements per field buffer
   int64_t spec_total = 0;   // complex elements per spectrum slot
-  LineCfg cfg_fx, cfg_y, cfg_z, cfg_zonly, cfg_ix;   // generic kernels: launches that cover every box
+  LineCfg cfg_x, cfg_y, cfg_z, cfg_zonly;   // generic kernels: launches that cover every box
   int smem_pf = 0, smem_pi = 0, smem_zf = 0;
-  int smem_penx = 0, smem_penxi = 0, smem_penc = 0, smem_penz = 0;
   int buf_pf = 0, buf_pi = 0, rows_pi = 0;     // complex elements per plane buffer
   int grid_pf = 0, grid_pi = 0;                // persistent grid sizes
   int reg_z = 0;                               // register z kernel length (0: none)
   int reg_zst = 0;                             // n1 * (n0/2 + 1) of every register-z box, else 0
   int z_prefetch = 64;                         // register z kernel: L2 prefetch distance in CTAs (64: measured
                                                // best of 0 .. 1216 on 512 boxes of 96^3)
-  int pen_rows_kb = 64;                        // pencil x pass: shared memory for one CTA's rows
   int host_copy = 1;                           // host path: 1 = SM copy kernel on mapped memory, 0 = copy engines
   int z_tile = 0;                              // plane/pencil z tile columns (0: the kernel maximum)
   // absorbing layers (form kPml): the description, boxes with layer cells,
@@ -438,11 +436,10 @@ struct psatd_plan {
   ShapeDev* d_shapes = nullptr;
   RowJob* d_rows_all = nullptr;
   ColJob *d_ycols_all = nullptr, *d_zcols = nullptr;
-  RowJob *d_g_rows = nullptr, *d_g_rows_int = nullptr;
-  ColJob *d_g_ycols = nullptr, *d_g_ycols_int = nullptr, *d_g_zcols = nullptr, *d_zfast = nullptr;
+  RowJob* d_g_rows_int = nullptr;
+  ColJob *d_g_ycols_int = nullptr, *d_g_zcols = nullptr, *d_zfast = nullptr;
   int2 *d_plane_fwd = nullptr, *d_plane_inv = nullptr;
-  RowJob *d_pen_rows = nullptr, *d_pen_rows_int = nullptr;
-  ColJob *d_pen_ycols = nullptr, *d_pen_ycols_int = nullptr, *d_zpen = nullptr, *d_zpen_reg = nullptr;
+  ColJob* d_zpen_reg = nullptr;
   CopyBlk* d_blocks = nullptr;
   XTile* d_tiles = nullptr;
   XTile* d_step_tiles = nullptr;
@@ -675,7 +672,7 @@ static void build_gather(psatd_plan* P, const std::vector<char>& box_fast, uint3
   P->deferred = false;
   const int nb = (int)P->boxes.size();
   const bool reg = !P->grp_pf.empty() && P->grp_pf.front().code >= 0 && !P->segs.empty() && P->step_tiles.empty() &&
-                   P->g_rows.empty() && P->pen_rows.empty() &&
+                   P->g_nrows == 0 &&
                    std::all_of(box_fast.begin(), box_fast.end(), [](char f) { return f != 0; });
   const bool pen = P->pen_boxes == nb && !P->step_tiles.empty();
   if ((flags & PSATD_EAGER_EXCHANGE) || !(reg || pen)) return;
@@ -742,7 +739,8 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
     s.L = b.n[0] / 2;
     s.hx = s.L + 1;
     s.p = b.order_p;
-    if (!line_plan(s.L, s.ax) || !line_plan(b.n[1], s.ay) || !line_plan(b.n[2], s.az))
+    if (!line_plan(s.L, s.ax, P->prec, true) || !line_plan(b.n[1], s.ay, P->prec, false) ||
+        !line_plan(b.n[2], s.az, P->prec, false))
       return fail(nullptr, PSATD_ERR_UNSUPPORTED_SIZE, "no radix schedule");
     s.ax.tw = tw_offset(s.L);
     s.ay.tw = tw_offset(b.n[1]);
@@ -798,6 +796,8 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
     gplane += b.n[2];
     x.foff = foff;
     x.soff = soff;
+    x.scale64 = 1.0 / ((double)b.n[0] * b.n[1] * b.n[2]);
+    x.scale32 = (float)x.scale64;
     foff += align_up((int64_t)b.n[0] * b.n[1] * b.n[2], 64);
     soff += align_up((int64_t)(b.n[0] / 2 + 1) * b.n[1] * b.n[2], 32);
     P->hboxes.push_back(x);
@@ -837,15 +837,30 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
     const int n2 = b.n[2], szf = z_fast_smem(P->prec, P->form, n2);
     const bool zr = z_reg_ok(n2) && z_reg_smem(P->form, n2) <= optin;
     const bool zf = sh.fz >= 0 && szf <= optin;
-    const bool zp = sh.pz >= 0 && n2 <= pen_z_max(P->prec) && szf <= optin;
+    const bool zp = sh.pz >= 0 && n2 <= pencil_max_z(P->prec) && szf <= optin;
     if (!(zr || zf || zp)) return -1;
     P->reg_planes_used = true;
     return P->reg_planes ? c : -1;
   };
   std::vector<int> box_reg(P->boxes.size(), -1);
-  std::vector<char> box_generic(P->boxes.size(), 0);
-  int64_t zcolumns = 0;          // z columns of the generic boxes
-  int zlongest = 0, zany = 0;    // their longest z line, and any box's
+  // the z pass of a box without a plane z kernel: the register z kernel of its
+  // length, in its own tiles (FP32, pencil-family boxes), else the generic one
+  std::vector<int> zgen;
+  auto z_boxes = [&](int bi, bool family) {
+    const psatd_box& b = P->boxes[bi];
+    if (P->prec == 32 && family) P->pen_reg_z_used = true;
+    if (P->prec == 32 && family && P->pen_reg_z && z_reg_ok(b.n[2]) && z_reg_smem(P->form, b.n[2]) <= optin &&
+        z_reg_multi_smem(P->form) <= optin) {
+      const int L = b.n[0] / 2, n1 = b.n[1], rt = z_reg_tile_width(P->form, b.n[2]);
+      for (int y = 0; y < n1; ++y)
+        for (int m = 0; m < L; m += rt) P->zpen_reg.push_back({bi, y, m, std::min(rt, L - m)});
+      for (int y = 0; y < n1; y += rt) P->zpen_reg.push_back({bi, y, L, -std::min(rt, n1 - y)});
+    } else {
+      zgen.push_back(bi);
+    }
+  };
+  std::vector<RowJob> fast_rows;
+  std::vector<ColJob> fast_ycols;
   for (int bi = 0; bi < (int)P->boxes.size(); ++bi) {
     const psatd_box& b = P->boxes[bi];
     const int n0 = b.n[0], n1 = b.n[1], n2 = b.n[2];
@@ -857,17 +872,14 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
     const bool fast_ok = plane_ok(b, sh);
     const int rows = n1 * n2;
     const int nr = line_tile_width(P->prec);
-    for (int r = 0; r < rows; r += nr) P->rows_all.push_back({bi, r, std::min(nr, rows - r), 0});
     const bool pencil_ok = !(d.flags & PSATD_GENERIC_KERNELS) && P->form != kPml && sh.px >= 0 && sh.py >= 0 &&
                            sh.pz >= 0 &&
-                           n2 <= pen_z_max(P->prec) && sm_zf <= optin && pen_col_smem(P->prec, n1) <= optin;
+                           n2 <= pencil_max_z(P->prec) && sm_zf <= optin;
     box_reg[bi] = reg_code_of(b, sh);
     const bool prefer_pencil =
         (d.flags & PSATD_PENCIL_KERNELS) || (!(d.flags & PSATD_PLANE_KERNELS) && box_reg[bi] < 0);
     const bool fast = (fast_ok || box_reg[bi] >= 0) && !(pencil_ok && prefer_pencil);
     const bool pencil = !fast && pencil_ok;
-    const bool generic = !fast && !pencil;   // the generic kernels
-    box_generic[bi] = generic;
     if (fast) {
       ++P->fast_boxes;
       for (int z = 0; z < n2; ++z) {
@@ -875,81 +887,64 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
         if (z >= b.ng_lo[2] && z < n2 - b.ng_hi[2]) P->plane_inv.push_back(make_int2(bi, z));
       }
       // z pass: the shared-memory plane z kernel (or the register z kernel,
-      // chosen below) where the z length has one, else the pencil z kernel
-      const bool zf = sh.fz >= 0 && sm_zf <= optin;
-      std::vector<ColJob>& zl = zf ? P->zfast : P->zpen;
-      for (int y = 0; y < n1; ++y)
-        for (int m = 0; m < L; m += tile) zl.push_back({bi, y, m, std::min(tile, L - m)});
-      // the Nyquist column mx = L in tiles of consecutive y (negative count)
-      for (int y = 0; y < n1; y += tile) zl.push_back({bi, y, L, -std::min(tile, n1 - y)});
-      if (zf)
+      // chosen below) where the z length has one, else the generic z pass
+      // (or its own register z kernel)
+      if (sh.fz >= 0 && sm_zf <= optin) {
+        for (int y = 0; y < n1; ++y)
+          for (int m = 0; m < L; m += tile) P->zfast.push_back({bi, y, m, std::min(tile, L - m)});
+        // the Nyquist column mx = L in tiles of consecutive y (negative count)
+        for (int y = 0; y < n1; y += tile) P->zfast.push_back({bi, y, L, -std::min(tile, n1 - y)});
         P->smem_zf = std::max(P->smem_zf, sm_zf);
-      else
-        P->smem_penz = std::max(P->smem_penz, sm_zf);
+      } else {
+        z_boxes(bi, true);
+      }
       if (fast_ok) {   // buffers of the shared-memory plane kernels
         P->buf_pf = std::max(P->buf_pf, n1 * sh.lp);
         P->buf_pi = std::max(P->buf_pi, n1 * hx);
         P->rows_pi = std::max(P->rows_pi, ni * sh.hp);
       }
-    } else if (pencil) {
-      // pencil kernels: x rows, y tiles, z tiles (+ update), y tiles, x rows
-      ++P->pen_boxes;
-      const int pr = pen_rows(P->prec, L, rows, P->pen_rows_kb * 1024);
-      for (int r = 0; r < rows; r += pr) P->pen_rows.push_back({bi, r, std::min(pr, rows - r), 0});
-      const int y0 = b.ng_lo[1], y1 = n1 - b.ng_hi[1];
-      const int pri = pen_rows(P->prec, L, y1 - y0, P->pen_rows_kb * 1024);
-      for (int z = b.ng_lo[2]; z < n2 - b.ng_hi[2]; ++z)
-        for (int y = y0; y < y1; y += pri) P->pen_rows_int.push_back({bi, z * n1 + y, std::min(pri, y1 - y), 0});
-      const int ct = pen_col_tile(P->prec);
-      for (int z = 0; z < n2; ++z)
-        for (int m = 0; m < hx; m += ct) {
-          const ColJob j{bi, z, m, std::min(ct, hx - m)};
-          P->pen_ycols.push_back(j);
-          if (z >= b.ng_lo[2] && z < n2 - b.ng_hi[2]) P->pen_ycols_int.push_back(j);
-        }
-      for (int y = 0; y < n1; ++y)
-        for (int m = 0; m < L; m += tile) P->zpen.push_back({bi, y, m, std::min(tile, L - m)});
-      for (int y = 0; y < n1; y += tile) P->zpen.push_back({bi, y, L, -std::min(tile, n1 - y)});
-      P->smem_penx = std::max(P->smem_penx, pen_x_smem(P->prec, L, pr));
-      P->smem_penxi = std::max(P->smem_penxi, pen_x_smem(P->prec, L, pri));
-      P->smem_penc = std::max(P->smem_penc, pen_col_smem(P->prec, n1));
-      P->smem_penz = std::max(P->smem_penz, sm_zf);
     } else {
-      for (int r = 0; r < rows; r += nr) P->g_rows.push_back({bi, r, std::min(nr, rows - r), 0});
+      if (pencil) ++P->pen_boxes;
+      z_boxes(bi, pencil);
       for (int z = b.ng_lo[2]; z < n2 - b.ng_hi[2]; ++z) {
         const int y0 = b.ng_lo[1], y1 = n1 - b.ng_hi[1];
         for (int y = y0; y < y1; y += nr) P->g_rows_int.push_back({bi, z * n1 + y, std::min(nr, y1 - y), 0});
       }
     }
-    line_cover(P->cfg_fx, P->prec, sh.ax, 1);
-    line_cover(P->cfg_ix, P->prec, sh.ax, 2);
-    line_cover(P->cfg_y, P->prec, sh.ay, 0);
-    line_cover(P->cfg_zonly, P->prec, sh.az, 0);
+    line_cover(P->cfg_x, P->prec, sh.ax, true);
+    line_cover(P->cfg_y, P->prec, sh.ay, false);
+    line_cover(P->cfg_zonly, P->prec, sh.az, false);
     // column tiles run on through the planes
-    const int yi0 = b.ng_lo[2], yi1 = n2 - b.ng_hi[2];
-    column_tiles(P->ycols_all, bi, 0, n2, hx, nr);
+    std::vector<RowJob>& rl = fast ? fast_rows : P->rows_all;
+    for (int r = 0; r < rows; r += nr) rl.push_back({bi, r, std::min(nr, rows - r), 0});
+    column_tiles(fast ? fast_ycols : P->ycols_all, bi, 0, n2, hx, nr);
     column_tiles(P->zcols, bi, 0, n1, hx, nr);
-    if (generic) {
-      column_tiles(P->g_ycols, bi, 0, n2, hx, nr);
-      column_tiles(P->g_ycols_int, bi, yi0, yi1, hx, nr);
-      zcolumns += (int64_t)n1 * hx;
-      zlongest = std::max(zlongest, n2);
-    }
+    if (!fast) column_tiles(P->g_ycols_int, bi, b.ng_lo[2], n2 - b.ng_hi[2], hx, nr);
   }
+  P->g_nrows = (int64_t)P->rows_all.size();
+  P->g_nycols = (int64_t)P->ycols_all.size();
+  P->rows_all.insert(P->rows_all.end(), fast_rows.begin(), fast_rows.end());
+  P->ycols_all.insert(P->ycols_all.end(), fast_ycols.begin(), fast_ycols.end());
   // the generic z pass: its tile width follows the longest line and the number of columns
-  for (const psatd_box& b : P->boxes) zany = std::max(zany, b.n[2]);
-  z_cover(P->cfg_z, P->prec, P->form, zlongest ? zlongest : zany, zlongest ? zcolumns : INT64_MAX, P->sms, optin);
-  for (const psatd_box& b : P->boxes) {
-    AxisPlan a{};
-    line_plan(b.n[2], a);
-    if (std::max(a.r1, a.r2) > 16) P->cfg_z.cls = 1;
+  int64_t zcolumns = 0;
+  int zlongest = 0;
+  for (int bi : zgen) {
+    const psatd_box& b = P->boxes[bi];
+    zcolumns += (int64_t)b.n[1] * (b.n[0] / 2 + 1);
+    zlongest = std::max(zlongest, b.n[2]);
   }
-  for (int bi = 0; bi < (int)P->boxes.size(); ++bi)
-    if (box_generic[bi])
-      column_tiles(P->g_zcols, bi, 0, P->boxes[bi].n[1], P->boxes[bi].n[0] / 2 + 1, 1 << P->cfg_z.lg);
+  if (zgen.empty()) {   // (a distributed group still uses it)
+    zcolumns = INT64_MAX;
+    for (const psatd_box& b : P->boxes) zlongest = std::max(zlongest, b.n[2]);
+  }
+  z_cover(P->cfg_z, P->prec, P->form, zlongest, zcolumns, P->z_tile, P->sms, optin);
+  for (const ShapeDev& sh : P->hshapes)
+    if (std::max(sh.az.r1, sh.az.r2) > 16) P->cfg_z.cls = 1;
+  for (int bi : zgen)
+    column_tiles(P->g_zcols, bi, 0, P->boxes[bi].n[1], P->boxes[bi].n[0] / 2 + 1, 1 << P->cfg_z.lg);
   // pencil jobs grouped by the FFT length of the axis each kernel transforms
   // (one launch per group; boxes keep their order inside a group)
-  auto group = [&](auto& list, auto code_of, std::vector<psatd_plan::PenGroup>& groups) {
+  auto group = [&](auto& list, auto code_of, std::vector<psatd_plan::Group>& groups) {
     std::stable_sort(list.begin(), list.end(),
                      [&](const auto& a, const auto& b) { return code_of(a) < code_of(b); });
     for (int64_t i = 0; i < (int64_t)list.size(); ++i) {
@@ -959,28 +954,6 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
     }
   };
   auto shape_of_box = [&](int box) -> const ShapeDev& { return P->hshapes[P->hboxes[box].shape]; };
-  // FP32 pencil boxes whose z length has a register z kernel: that kernel
-  // does their z pass (z FFT, update, inverse z FFT), its jobs re-tiled to
-  // its own tile width; the shared-memory pencil z kernel keeps the rest
-  if (P->prec == 32 && !P->zpen.empty()) P->pen_reg_z_used = true;
-  if (P->prec == 32 && P->pen_reg_z && !P->zpen.empty()) {
-    std::vector<ColJob> keep;
-    std::vector<char> done(P->boxes.size(), 0);
-    for (const ColJob& j : P->zpen) {
-      const psatd_box& b = P->boxes[j.box];
-      if (!(z_reg_ok(b.n[2]) && z_reg_smem(P->form, b.n[2]) <= optin && z_reg_multi_smem(P->form) <= optin)) {
-        keep.push_back(j);
-        continue;
-      }
-      if (done[j.box]) continue;
-      done[j.box] = 1;
-      const int L = b.n[0] / 2, n1 = b.n[1], rt = z_reg_tile_width(P->form, b.n[2]);
-      for (int y = 0; y < n1; ++y)
-        for (int m = 0; m < L; m += rt) P->zpen_reg.push_back({j.box, y, m, std::min(rt, L - m)});
-      for (int y = 0; y < n1; y += rt) P->zpen_reg.push_back({j.box, y, L, -std::min(rt, n1 - y)});
-    }
-    P->zpen.swap(keep);
-  }
   if (P->fast_boxes && P->prec == 32) {
     // register plane kernels for the fast boxes with a register shape: the
     // plane jobs grouped by shape (one launch each), box order kept in a
@@ -1026,11 +999,6 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
   P->zreg_multi = !P->zpen_reg.empty() && std::all_of(P->grp_zreg.begin(), P->grp_zreg.end(), [](const auto& g) {
     return z_reg_multi_ok(g.code) != 0;
   });
-  group(P->pen_rows, [&](const RowJob& j) { return shape_of_box(j.box).px; }, P->grp_rows);
-  group(P->pen_rows_int, [&](const RowJob& j) { return shape_of_box(j.box).px; }, P->grp_rows_int);
-  group(P->pen_ycols, [&](const ColJob& j) { return shape_of_box(j.box).py; }, P->grp_ycols);
-  group(P->pen_ycols_int, [&](const ColJob& j) { return shape_of_box(j.box).py; }, P->grp_ycols_int);
-  group(P->zpen, [&](const ColJob& j) { return shape_of_box(j.box).pz; }, P->grp_z);
   if (P->fast_boxes && P->prec == 32 && !P->zfast.empty()) {
     // one register z length for every fast box, or none
     int nz = -2;
@@ -1135,19 +1103,12 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
   CK(P, upload(P, P->rows_all, &P->d_rows_all));
   CK(P, upload(P, P->ycols_all, &P->d_ycols_all));
   CK(P, upload(P, P->zcols, &P->d_zcols));
-  CK(P, upload(P, P->g_rows, &P->d_g_rows));
   CK(P, upload(P, P->g_rows_int, &P->d_g_rows_int));
-  CK(P, upload(P, P->g_ycols, &P->d_g_ycols));
   CK(P, upload(P, P->g_ycols_int, &P->d_g_ycols_int));
   CK(P, upload(P, P->g_zcols, &P->d_g_zcols));
   CK(P, upload(P, P->zfast, &P->d_zfast));
   CK(P, upload(P, P->plane_fwd, &P->d_plane_fwd));
   CK(P, upload(P, P->plane_inv, &P->d_plane_inv));
-  CK(P, upload(P, P->pen_rows, &P->d_pen_rows));
-  CK(P, upload(P, P->pen_rows_int, &P->d_pen_rows_int));
-  CK(P, upload(P, P->pen_ycols, &P->d_pen_ycols));
-  CK(P, upload(P, P->pen_ycols_int, &P->d_pen_ycols_int));
-  CK(P, upload(P, P->zpen, &P->d_zpen));
   CK(P, upload(P, P->zpen_reg, &P->d_zpen_reg));
   CK(P, upload(P, P->blocks, &P->d_blocks));
   CK(P, upload(P, P->tiles, &P->d_tiles));
@@ -1218,14 +1179,13 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   free_tmp();
   CK(P, e);
-  const int smem = std::max({P->cfg_fx.smem, P->cfg_y.smem, P->cfg_z.smem, P->cfg_zonly.smem, P->cfg_ix.smem, P->smem_pf,
-                             P->smem_pi, P->smem_zf, P->smem_penx, P->smem_penxi, P->smem_penc, P->smem_penz});
+  const int smem = std::max({P->cfg_x.smem, P->cfg_y.smem, P->cfg_z.smem, P->cfg_zonly.smem, P->smem_pf,
+                             P->smem_pi, P->smem_zf});
   if (smem > optin) return fail(P, PSATD_ERR_UNSUPPORTED_SIZE, fmt("needs %d B shared memory", smem));
   // The attribute is a per-kernel cap shared by every plan: raise it to the
   // device maximum so that no plan lowers it below another plan's need.
   CK(P, configure_kernels(P->prec, optin));
   CK(P, configure_fast_kernels(P->prec, optin));
-  CK(P, configure_pen_kernels(P->prec, optin));
   if (P->prec == 32) CK(P, configure_reg_kernels(optin));
   if (P->fast_boxes) {
     int sms = 0, occ_f = 0, occ_i = 0;
@@ -1566,7 +1526,6 @@ psatd_status psatd_plan_create(const psatd_plan_desc* desc, void* stream, psatd_
     for (int i = 0; desc->tuning && i < 16 && desc->tuning[2 * i] != 0; ++i) {
       const int32_t k = desc->tuning[2 * i], v = desc->tuning[2 * i + 1];
       if (k == PSATD_TUNE_Z_PREFETCH) P->z_prefetch = v;
-      if (k == PSATD_TUNE_PENCIL_ROWS_KB) P->pen_rows_kb = v;
       if (k == PSATD_TUNE_Z_TILE) P->z_tile = v;
       if (k == PSATD_TUNE_HOST_COPY) P->host_copy = v;
       if (k == PSATD_TUNE_PENCIL_REG_Z) P->pen_reg_z = v;
@@ -1688,7 +1647,7 @@ static psatd_status forward_xy(psatd_plan* P, const DevPlan& D, const FieldPtrs&
                                cudaStream_t st, int64_t* launches_out, bool gather = false) {
   const int64_t S = P->spec_total;
   int64_t launches = 0;
-  // fast boxes: one plane kernel; generic: x rows, y columns; pencil: x rows, y tiles
+  // fast boxes: one plane kernel; generic and pencil boxes: x rows, y columns
   if (!P->grp_pf.empty()) {
     // one launch per register plane shape; the gather tables are indexed by plane_fwd position
     for (const auto& g : P->grp_pf) {
@@ -1715,29 +1674,15 @@ static psatd_status forward_xy(psatd_plan* P, const DevPlan& D, const FieldPtrs&
        }));
     ++launches;
   }
-  if (!P->g_rows.empty()) {
+  if (P->g_nrows) {
     CK(P, timed(P, 0, st, [&] {
-         return launch_fwd_x(P->prec, D, fp, nf, spec, S, P->d_g_rows, (int64_t)P->g_rows.size(), P->cfg_fx, st);
+         return launch_fwd_x(P->prec, D, fp, nf, spec, S, P->d_rows_all, P->g_nrows, P->cfg_x,
+                             gather && !P->ggrid.empty() ? P->d_ggrid : nullptr, fields_out(P->form), st);
        }));
     CK(P, timed(P, 1, st, [&] {
-         return launch_col(P->prec, -1, 1, D, spec, S, nf, P->d_g_ycols, (int64_t)P->g_ycols.size(), P->cfg_y, st);
+         return launch_col(P->prec, -1, 1, D, spec, S, nf, P->d_ycols_all, P->g_nycols, P->cfg_y, st);
        }));
     launches += 2;
-  }
-  for (const auto& g : P->grp_rows) {
-    CK(P, timed(P, 0, st, [&] {
-         return launch_pen_xf(P->prec, g.code, D, fp, nf, spec, S, P->d_pen_rows + g.start, g.count, P->smem_penx,
-                              gather && P->deferred && !P->ggrid.empty() ? P->d_ggrid : nullptr, fields_out(P->form),
-                              st);
-       }));
-    ++launches;
-  }
-  for (const auto& g : P->grp_ycols) {
-    CK(P, timed(P, 1, st, [&] {
-         return launch_pen_col(P->prec, -1, g.code, D, spec, S, nf, P->d_pen_ycols + g.start, g.count,
-                               P->smem_penc, st);
-       }));
-    ++launches;
   }
   *launches_out += launches;
   return PSATD_OK;
@@ -1763,7 +1708,7 @@ static psatd_status transform_current(psatd_plan* P, const DevPlan& D, const Fie
   // every box's z pass is a thread-pair register z kernel with 8-column tiles,
   // else the generic column kernel
   const int rt = z_reg_tile_width(P->form, P->reg_z ? P->reg_z : 48);
-  const bool zreg = P->prec == 32 && P->zpen.empty() && P->g_zcols.empty() && rt == 8 &&
+  const bool zreg = P->prec == 32 && P->g_zcols.empty() && rt == 8 &&
                     (P->zfast.empty() || (P->reg_z && z_reg_multi_ok(P->reg_z))) &&
                     std::all_of(P->grp_zreg.begin(), P->grp_zreg.end(),
                                 [](const auto& g) { return z_reg_multi_ok(g.code) != 0; }) &&
@@ -1807,17 +1752,10 @@ static psatd_status z_step(psatd_plan* P, const DevPlan& D, cudaStream_t st, int
        }));
     ++launches;
   }
-  for (const auto& g : one_launch ? std::vector<psatd_plan::PenGroup>() : P->grp_zreg) {
+  for (const auto& g : one_launch ? std::vector<psatd_plan::Group>() : P->grp_zreg) {
     CK(P, timed(P, 2, st, [&] {
          return launch_z_reg(P->form, D, P->d_ws, S, P->d_zpen_reg + g.start, g.count, g.code, 0, NFT, P->z_prefetch,
                              st);
-       }));
-    ++launches;
-  }
-  for (const auto& g : P->grp_z) {
-    CK(P, timed(P, 2, st, [&] {
-         return launch_z_pen(P->prec, P->form, g.code, D, P->d_ws, S, P->d_zpen + g.start, g.count, P->smem_penz,
-                             NFT, st);
        }));
     ++launches;
   }
@@ -1882,28 +1820,14 @@ static psatd_status inverse_step(psatd_plan* P, const DevPlan& D, const FieldPtr
        }));
     ++launches;
   }
-  if (!P->g_rows.empty()) {
+  if (P->g_nrows) {
     CK(P, timed(P, 3, st, [&] {
          return launch_col(P->prec, 1, 1, D, spec, S, nout, P->d_g_ycols_int, (int64_t)P->g_ycols_int.size(), P->cfg_y, st);
        }));
     CK(P, timed(P, 4, st, [&] {
-         return launch_inv_x(P->prec, D, fp, nout, spec, S, P->d_g_rows_int, (int64_t)P->g_rows_int.size(), P->cfg_ix, 1, st);
+         return launch_inv_x(P->prec, D, fp, nout, spec, S, P->d_g_rows_int, (int64_t)P->g_rows_int.size(), P->cfg_x, 1, st);
        }));
     launches += 2;
-  }
-  for (const auto& g : P->grp_ycols_int) {
-    CK(P, timed(P, 3, st, [&] {
-         return launch_pen_col(P->prec, 1, g.code, D, spec, S, nout, P->d_pen_ycols_int + g.start, g.count,
-                               P->smem_penc, st);
-       }));
-    ++launches;
-  }
-  for (const auto& g : P->grp_rows_int) {
-    CK(P, timed(P, 4, st, [&] {
-         return launch_pen_xi(P->prec, g.code, D, fp, nout, spec, S, P->d_pen_rows_int + g.start, g.count,
-                              P->smem_penxi, st);
-       }));
-    ++launches;
   }
   if (P->form == kPml && !P->pml_boxes.empty()) {
     // absorbing layers, step (2): damp the split parts, rebuild the components
@@ -2249,7 +2173,7 @@ psatd_status psatd_forward_fft(psatd_plan* P, const void* field, void* spectrum,
   P->last_stream = st;
   const DevPlan D = P->dev();
   const int64_t S = P->spec_total;
-  CK(P, launch_fwd_x(P->prec, D, fp, 1, spectrum, S, P->d_rows_all, (int64_t)P->rows_all.size(), P->cfg_fx, st));
+  CK(P, launch_fwd_x(P->prec, D, fp, 1, spectrum, S, P->d_rows_all, (int64_t)P->rows_all.size(), P->cfg_x, nullptr, 0, st));
   CK(P, launch_col(P->prec, -1, 1, D, spectrum, S, 1, P->d_ycols_all, (int64_t)P->ycols_all.size(), P->cfg_y, st));
   CK(P, launch_col(P->prec, -1, 2, D, spectrum, S, 1, P->d_zcols, (int64_t)P->zcols.size(), P->cfg_zonly, st));
   P->last_launches = 3;
@@ -2268,7 +2192,7 @@ psatd_status psatd_inverse_fft(psatd_plan* P, void* spectrum, void* field, void*
   const int64_t S = P->spec_total;
   CK(P, launch_col(P->prec, 1, 2, D, spectrum, S, 1, P->d_zcols, (int64_t)P->zcols.size(), P->cfg_zonly, st));
   CK(P, launch_col(P->prec, 1, 1, D, spectrum, S, 1, P->d_ycols_all, (int64_t)P->ycols_all.size(), P->cfg_y, st));
-  CK(P, launch_inv_x(P->prec, D, fp, 1, spectrum, S, P->d_rows_all, (int64_t)P->rows_all.size(), P->cfg_ix, 0, st));
+  CK(P, launch_inv_x(P->prec, D, fp, 1, spectrum, S, P->d_rows_all, (int64_t)P->rows_all.size(), P->cfg_x, 0, st));
   P->last_launches = 3;
   return PSATD_OK;
 }
@@ -2364,7 +2288,7 @@ psatd_status psatd_dist_forward_xy(psatd_plan* P, const psatd_fields* slab, cons
   DevPlan D = P->dev();
   D.boxes = P->dist.d_boxes;
   const auto& d = P->dist;
-  CK(P, launch_fwd_x(P->prec, D, fp, nf, slab_spectrum, d.s_slab, d.d_rows, d.nrows, P->cfg_fx, st));
+  CK(P, launch_fwd_x(P->prec, D, fp, nf, slab_spectrum, d.s_slab, d.d_rows, d.nrows, P->cfg_x, nullptr, 0, st));
   CK(P, launch_col(P->prec, -1, 1, D, slab_spectrum, d.s_slab, nf, d.d_ycols, d.nycols, P->cfg_y, st));
   P->last_launches = 2;
   return PSATD_OK;
@@ -2402,7 +2326,7 @@ psatd_status psatd_dist_inverse_yx(psatd_plan* P, void* slab_spectrum, const psa
   D.boxes = P->dist.d_boxes;
   const auto& d = P->dist;
   CK(P, launch_col(P->prec, 1, 1, D, slab_spectrum, d.s_slab, FOUT, d.d_ycols, d.nycols, P->cfg_y, st));
-  CK(P, launch_inv_x(P->prec, D, fp, FOUT, slab_spectrum, d.s_slab, d.d_rows, d.nrows, P->cfg_ix, 1, st));
+  CK(P, launch_inv_x(P->prec, D, fp, FOUT, slab_spectrum, d.s_slab, d.d_rows, d.nrows, P->cfg_x, 1, st));
   P->last_launches = 2;
   return PSATD_OK;
 }
@@ -2486,7 +2410,7 @@ int32_t psatd_plan_tuning(const psatd_plan* P, int32_t knob) {
     case PSATD_TUNE_Z_PREFETCH:
       return P->reg_z || !P->zpen_reg.empty() ? P->z_prefetch : -1;
     case PSATD_TUNE_PENCIL_ROWS_KB:
-      return P->pen_boxes ? P->pen_rows_kb : -1;
+      return -1;   // accepted, used by no kernel
     case PSATD_TUNE_HOST_COPY:
       return P->host_copy;
     case PSATD_TUNE_PENCIL_REG_Z:

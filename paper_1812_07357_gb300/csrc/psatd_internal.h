@@ -67,9 +67,9 @@ struct ShapeDev {
   X(5, 60, 12, 5) X(6, 64, 8, 8) X(7, 80, 10, 8) X(8, 96, 12, 8) X(9, 120, 12, 10)       \
   X(10, 128, 16, 8)
 
-// Lengths of the pencil kernels (boxes too large for the plane kernels):
-// the same two-pass factorizations, extended to 512.  Codes 0-10 coincide
-// with PSATD_FAST_LENGTHS.
+// Lengths of the pencil family (boxes too large for the plane kernels, on the
+// generic kernels with the deferred exchange and the register z kernels); z
+// lengths up to pencil_max_z.  Codes 0-10 coincide with PSATD_FAST_LENGTHS.
 #define PSATD_PENCIL_LENGTHS(X)                                                         \
   PSATD_FAST_LENGTHS(X)                                                                \
   X(11, 144, 12, 12) X(12, 160, 16, 10) X(13, 192, 16, 12) X(14, 240, 24, 10)            \
@@ -82,6 +82,8 @@ inline int pencil_code(int n) {
 #undef PSATD_CODE
   return -1;
 }
+
+inline int pencil_max_z(int prec) { return prec == 32 ? 256 : 128; }
 
 inline int fast_code(int n) {
 #define PSATD_CODE(code, N, R1, R2) \
@@ -100,6 +102,9 @@ struct BoxDev {
   int32_t yoff;                   // global index of the box's spectrum row my = 0 (rows of a distributed group)
   int64_t foff;                   // element offset in every field buffer
   int64_t soff;                   // complex-element offset in every spectrum slot
+  double scale64;                 // 1 / (n0 n1 n2), the inverse transform's factor
+  float scale32;                  // ... rounded once
+  int32_t pad;
 };
 
 // rows r0 .. r0+nr-1 of one box, row r = y + n1*z (x-axis passes)
@@ -189,12 +194,15 @@ inline void set_constants(DevPlan& P, double c, double eps0, double dt) {
   P.icce = 1.0 / (c * c * eps0);
 }
 
-// ---- generic kernels (fft_kernels.cu, any_z.cu) ---------------------------
+// ---- generic kernels (fft_kernels.cu, any_lines.cuh, any_z.cuh) ---------------------------
 
 // Forward R2C along x of `nf` field slots into spectrum slots (stride
 // sstride); row jobs of at most line_tile_width rows.
+// ggrid (deferred exchange): the gather grid of every plane, box b's plane z
+// at boxes[b].gplane + z, used for the slots f < ngather; null: plain rows
 cudaError_t launch_fwd_x(int prec, const DevPlan& P, const FieldPtrs& f, int nf, void* spec, int64_t sstride,
-                         const RowJob* jobs, int64_t njobs, const LineCfg& c, cudaStream_t st);
+                         const RowJob* jobs, int64_t njobs, const LineCfg& c, const GatherGrid* ggrid, int ngather,
+                         cudaStream_t st);
 // Complex FFT along y (axis 1) or z (axis 2), in place on spectrum slots;
 // column jobs of at most line_tile_width columns.
 cudaError_t launch_col(int prec, int dir, int axis, const DevPlan& P, void* spec, int64_t sstride, int nf,
@@ -208,9 +216,8 @@ cudaError_t launch_z_update(int prec, int form, const DevPlan& P, void* spec, in
 cudaError_t launch_inv_x(int prec, const DevPlan& P, const FieldPtrs& f, int nf, void* spec, int64_t sstride,
                          const RowJob* jobs, int64_t njobs, const LineCfg& c, int interior_only, cudaStream_t st);
 int line_tile_width(int prec);   // rows or columns of a tile
-void line_cover(LineCfg& c, int prec, const AxisPlan& a, int kind);
-void z_cover(LineCfg& c, int prec, int form, int n2_max, int64_t columns, int sms, int optin);
-cudaError_t configure_any_z(int prec, int smem_bytes);
+void line_cover(LineCfg& c, int prec, const AxisPlan& a, bool rows);
+void z_cover(LineCfg& c, int prec, int form, int n2_max, int64_t columns, int widest, int sms, int optin);
 
 // ---- exchange (exchange.cu) -------------------------------------------------
 // Guard exchange of `nf` field slots.
@@ -319,30 +326,11 @@ cudaError_t launch_z_reg_multi(int form, const DevPlan& P, void* spec, int64_t s
                                int64_t njobs, int grid, int prefetch, int nft, cudaStream_t st);
 int z_reg_multi_smem(int form);
 
-// ---- pencil kernels (pencil_kernels.cu): boxes of two-pass lengths too large
-// for the plane kernels; the z pass takes fast_tile(prec) mx columns per tile
-int pen_rows(int prec, int L, int rows, int smem_cap);   // x rows per CTA
-int pen_x_smem(int prec, int L, int nr);
-int pen_z_max(int prec);                                  // longest n2 of a pencil box
-int pen_col_tile(int prec);                               // mx columns of a y tile
-int pen_col_smem(int prec, int n1);
-// one launch per length group: `code` = pencil code of the transformed axis
-// ggrid (deferred exchange): the gather grid of every plane, box b's plane z
-// at boxes[b].gplane + z, used for the slots f < ngather; null: plain rows
-cudaError_t launch_pen_xf(int prec, int code, const DevPlan& P, const FieldPtrs& f, int nf, void* spec,
-                          int64_t sstride, const RowJob* jobs, int64_t njobs, int smem, const GatherGrid* ggrid, int ngather, cudaStream_t st);
-cudaError_t launch_pen_col(int prec, int dir, int code, const DevPlan& P, void* spec, int64_t sstride, int nf,
-                           const ColJob* jobs, int64_t njobs, int smem, cudaStream_t st);
-cudaError_t launch_z_pen(int prec, int form, int code, const DevPlan& P, void* spec, int64_t sstride,
-                         const ColJob* jobs, int64_t njobs, int smem, int nft, cudaStream_t st);
-cudaError_t launch_pen_xi(int prec, int code, const DevPlan& P, const FieldPtrs& f, int nf, void* spec,
-                          int64_t sstride, const RowJob* jobs, int64_t njobs, int smem, cudaStream_t st);
-cudaError_t configure_pen_kernels(int prec, int smem_bytes);
-
 // ---- host helpers (plan.cpp) ------------------------------------------------
 // Two radices and the index maps of a complex FFT length (false when there are
-// none: not 5-smooth, or above 1024).
-bool line_plan(int n, AxisPlan& ap);
+// none: not 5-smooth, or above 1024).  row: an x line; FP32 rows take no
+// prime-factor maps (their lanes run along the row, which such maps scatter).
+bool line_plan(int n, AxisPlan& ap, int prec, bool row);
 // Tiles of `w` columns of the planes [p0, p1) of a box, hx columns each, the
 // columns numbered through the planes.
 void column_tiles(std::vector<ColJob>& out, int box, int p0, int p1, int hx, int w);

@@ -107,7 +107,7 @@ extern "C" psatd_status psatd_push_box_static(const int32_t n[3], int32_t order_
   s.L = L;
   s.hx = hx;
   s.p = order_p;
-  if (!line_plan(L, s.ax) || !line_plan(n1, s.ay) || !line_plan(n2, s.az))
+  if (!line_plan(L, s.ax, 32, true) || !line_plan(n1, s.ay, 32, false) || !line_plan(n2, s.az, 32, false))
     return err(PSATD_ERR_UNSUPPORTED_SIZE, "no radix schedule");
   int64_t ctot = 0, rtot = 0;
   auto ctake = [&](int64_t k) {
@@ -134,21 +134,22 @@ extern "C" psatd_status psatd_push_box_static(const int32_t n[3], int32_t order_
   const int64_t qtot = (int64_t)hx * (n1 / 2 + 1) * (n2 / 2 + 1);
   BoxDev b{};
   for (int a = 0; a < 3; ++a) b.n[a] = n[a];
+  b.scale64 = 1.0 / ((double)n0 * n1 * n2);
+  b.scale32 = (float)b.scale64;
   const int64_t spec = (int64_t)hx * n1 * n2;
   std::vector<RowJob> rows;
   std::vector<ColJob> ycols, zcols;
   const int nr = line_tile_width(32);
   for (int r = 0; r < n1 * n2; r += nr) rows.push_back({0, r, std::min(nr, n1 * n2 - r), 0});
   column_tiles(ycols, 0, 0, n2, hx, nr);
-  LineCfg cfx, cix, cy, cz;
-  line_cover(cfx, 32, s.ax, 1);
-  line_cover(cix, 32, s.ax, 2);
-  line_cover(cy, 32, s.ay, 0);
-  // two tiles per SM of the largest part, so that the lists do not depend on the device
-  z_cover(cz, 32, kVacuum, n2, (int64_t)n1 * hx, 160, 200 * 1024);
+  LineCfg cfx, cy, cz;
+  line_cover(cfx, 32, s.ax, true);
+  line_cover(cy, 32, s.ay, false);
+  // a tile per SM of the largest part, so that the lists do not depend on the device
+  z_cover(cz, 32, kVacuum, n2, (int64_t)n1 * hx, 0, 160, 200 * 1024);
   cz.cls = std::max(s.az.r1, s.az.r2) > 16;
   column_tiles(zcols, 0, 0, n1, hx, 1 << cz.lg);
-  const int smem = std::max({cfx.smem, cix.smem, cy.smem, cz.smem});
+  const int smem = std::max({cfx.smem, cy.smem, cz.smem});
   const std::vector<double> alpha = order_p ? stencil_alpha(order_p) : std::vector<double>(1, 0.0);
 
   // ---- carve the arena: [box][shape][rows][ycols][zcols][alpha][r32][c32][q32][r64][c64][q64][spectra]
@@ -251,11 +252,11 @@ extern "C" psatd_status psatd_push_box_static(const int32_t n[3], int32_t order_
   const ColJob* dy = reinterpret_cast<const ColJob*>(A + o_ycols);
   const ColJob* dz = reinterpret_cast<const ColJob*>(A + o_zcols);
   for (int step = 0; step < nsteps; ++step) {
-    PSATD_CK(launch_fwd_x(32, P, fp, FIN, ws, spec, drows, (int64_t)rows.size(), cfx, st));
+    PSATD_CK(launch_fwd_x(32, P, fp, FIN, ws, spec, drows, (int64_t)rows.size(), cfx, nullptr, 0, st));
     PSATD_CK(launch_col(32, -1, 1, P, ws, spec, FIN, dy, (int64_t)ycols.size(), cy, st));
     PSATD_CK(launch_z_update(32, kVacuum, P, ws, spec, dz, (int64_t)zcols.size(), cz, FIN, st));
     PSATD_CK(launch_col(32, 1, 1, P, ws, spec, FIN, dy, (int64_t)ycols.size(), cy, st));
-    PSATD_CK(launch_inv_x(32, P, fp, FIN, ws, spec, drows, (int64_t)rows.size(), cix, 1, st));
+    PSATD_CK(launch_inv_x(32, P, fp, FIN, ws, spec, drows, (int64_t)rows.size(), cfx, 1, st));
   }
 #undef PSATD_CK
   return PSATD_OK;
