@@ -1985,6 +1985,14 @@ static bool host_mapped(const psatd_plan* P, void* const host[6], void* const de
   return mapped;
 }
 
+// Blocks of the host copy kernel: 48 x 256 threads x 64 bytes = 0.8 MB in
+// flight covers the host link (211 GB/s at some 3 us).  With two blocks per SM
+// every kernel beside a copy was stretched to the length of the copy: its
+// misses queued behind the host reads of its SM.  A step of a 256 x 256 x 128
+// domain in 96^3 boxes: 304 blocks 2.98 ms, 152 2.93, 96 2.66, 64 2.63, 48 2.61,
+// 32 2.62, 24 2.72, 16 2.73.
+constexpr int kCopyBlocks = 48;
+
 // The host paths' transfers and push, component by component.  Component c
 // is copied between the host buffer src[c] / dst[c] and the device buffer
 // stage[c] (nbytes) on a side stream, by the copy kernel through the host
@@ -2000,9 +2008,6 @@ static psatd_status host_pipeline(psatd_plan* P, void* const src[6], void* const
   FieldPtrs hin{}, hout{}, dev_g{};
   const bool mapped = host_mapped(P, src, stage, nbytes, hin, dev_g) &&
                       host_mapped(P, dst, stage, nbytes, hout, dev_g);
-  int sms = 0, gpu = 0;
-  CK(P, cudaGetDevice(&gpu));
-  CK(P, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, gpu));
   // Component by component, the host copies on a side stream overlap the
   // scatter into the boxes and the forward x, y transforms of the previous
   // component (and, on the way back, the inverse y, x transforms and the
@@ -2028,7 +2033,7 @@ static psatd_status host_pipeline(psatd_plan* P, void* const src[6], void* const
       FieldPtrs h1{}, d1{};
       h1.p[0] = to_dev ? hin.p[c] : hout.p[c];
       d1.p[0] = stage[c];
-      return launch_copy_fields(to_dev ? d1 : h1, to_dev ? h1 : d1, 1, (int64_t)nbytes, 2 * sms, cs);
+      return launch_copy_fields(to_dev ? d1 : h1, to_dev ? h1 : d1, 1, (int64_t)nbytes, kCopyBlocks, cs);
     }
     return cudaMemcpyAsync(to_dev ? stage[c] : dst[c], to_dev ? src[c] : stage[c], nbytes,
                            to_dev ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToHost, cs);
@@ -2083,11 +2088,12 @@ static psatd_status host_pipeline(psatd_plan* P, void* const src[6], void* const
     launches += P->last_launches;
   }
   for (int c = 0; c < 6; ++c) {
-    // (split) the last step's inverse y, x transforms of component c, storing
-    // the guard cells; (with a coupling) its box interiors gathered back into
-    // the domain; to the host
+    // (split) the last step's inverse y, x transforms of component c; (with a
+    // coupling) its box interiors gathered back into the domain, which reads no
+    // guard cell (the next call's scatter fills them), else the guard cells
+    // stored too; to the host
     if (split) {
-      r = inverse_step(P, D, slot_fields(c), 1, slot_spec(c), st, &launches, true);
+      r = inverse_step(P, D, slot_fields(c), 1, slot_spec(c), st, &launches, !coupling);
       if (r != PSATD_OK) return r;
     }
     if (coupling) {
