@@ -44,6 +44,7 @@
 
 #include "any_fft.cuh"
 #include "fft_codelets.cuh"
+#include "launch.cuh"
 #include "psatd_internal.h"
 #include "psatd_update.cuh"
 
@@ -153,6 +154,7 @@ __global__ void __launch_bounds__(line_threads<T, CLS>())
   __shared__ RowBands<T> bands;
   const T* fb = reinterpret_cast<const T*>(F.p[f]);
   const bool gather = GATHER && f < ngather;
+  grid_order(P.order);
   if (gather) {
     if (threadIdx.x < J.nr) {
       const int t = threadIdx.x, r = J.r0 + t, n1 = bx.n[1], z = r / n1, y = r - z * n1;
@@ -248,6 +250,7 @@ __global__ void __launch_bounds__(line_threads<T, CLS>()) k_col(DevPlan P, cx<T>
   }
   cx<T>* g = spec + blockIdx.y * sstride + bx.soff + (int64_t)pl * (axis == 1 ? n1 * hx : hx) + m;
   cx<T>* col = reinterpret_cast<cx<T>*>(smem_raw) + c;   // place p of the column at col[p * W]
+  grid_order(P.order);
   if (live)
     with_radix<CLS>(l.r1, [&](auto rc) {
       for (int n2 = g0; n2 < l.r2; n2 += gs)
@@ -300,6 +303,7 @@ __global__ void __launch_bounds__(line_threads<T, CLS>(), sizeof(T) == 4 && !CLS
   const int nxi = (interior_only ? n0 - bx.ng_hi[0] : n0) - xlo;
   const bool pairs = ((xlo | nxi) & 1) == 0;   // whole pairs of cells
   const cx<T>* in = spec + f * sstride + bx.soff + (int64_t)J.r0 * hx;
+  grid_order(P.order);
   if constexpr (sizeof(T) == 4) {
     // lanes along the row: every thread merges its own samples from HBM (both
     // ends of a pair, the other end from L1) and stores its outputs to HBM

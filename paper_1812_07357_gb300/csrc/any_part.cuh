@@ -3,6 +3,7 @@
 #include "any_lines.cuh"
 #include "any_part.h"
 #include "any_z.cuh"
+#include "launch.cuh"
 
 namespace psatd {
 
@@ -12,9 +13,9 @@ void AnyPart<T, CLS>::fwd_x(dim3 grid, const DevPlan& P, const FieldPtrs& f, voi
                             cudaStream_t st) {
   cx<T>* s = static_cast<cx<T>*>(spec);
   if (ggrid)
-    k_fwd_x<T, CLS, true><<<grid, c.threads, c.smem, st>>>(P, f, s, sstride, jobs, ggrid, ngather);
+    launch_ordered(P.order, k_fwd_x<T, CLS, true>, grid, c.threads, c.smem, st, P, f, s, sstride, jobs, ggrid, ngather);
   else
-    k_fwd_x<T, CLS, false><<<grid, c.threads, c.smem, st>>>(P, f, s, sstride, jobs, ggrid, ngather);
+    launch_ordered(P.order, k_fwd_x<T, CLS, false>, grid, c.threads, c.smem, st, P, f, s, sstride, jobs, ggrid, ngather);
 }
 
 template <typename T, int CLS>
@@ -22,15 +23,15 @@ void AnyPart<T, CLS>::col(dim3 grid, int dir, int axis, const DevPlan& P, void* 
                           const ColJob* jobs, const LineCfg& c, cudaStream_t st) {
   cx<T>* s = static_cast<cx<T>*>(spec);
   if (dir < 0)
-    k_col<T, -1, CLS><<<grid, c.threads, c.smem, st>>>(P, s, sstride, axis, jobs);
+    launch_ordered(P.order, k_col<T, -1, CLS>, grid, c.threads, c.smem, st, P, s, sstride, axis, jobs);
   else
-    k_col<T, 1, CLS><<<grid, c.threads, c.smem, st>>>(P, s, sstride, axis, jobs);
+    launch_ordered(P.order, k_col<T, 1, CLS>, grid, c.threads, c.smem, st, P, s, sstride, axis, jobs);
 }
 
 template <typename T, int CLS>
 void AnyPart<T, CLS>::inv_x(dim3 grid, const DevPlan& P, const FieldPtrs& f, void* spec, int64_t sstride,
                             const RowJob* jobs, const LineCfg& c, int interior_only, cudaStream_t st) {
-  k_inv_x<T, CLS><<<grid, c.threads, c.smem, st>>>(P, f, static_cast<const cx<T>*>(spec), sstride, jobs,
+  launch_ordered(P.order, k_inv_x<T, CLS>, grid, c.threads, c.smem, st, P, f, static_cast<const cx<T>*>(spec), sstride, jobs,
                                                    interior_only);
 }
 
@@ -40,10 +41,10 @@ void AnyPart<T, CLS>::z_update(dim3 grid, int form, const DevPlan& P, void* spec
   cx<T>* s = static_cast<cx<T>*>(spec);
   constexpr int NT = z_threads<T>();
   switch (form) {
-    case kVacuum: k_z_update<T, kVacuum, CLS><<<grid, NT, c.smem, st>>>(P, s, sstride, jobs, nft, c.lg); break;
-    case kJForm: k_z_update<T, kJForm, CLS><<<grid, NT, c.smem, st>>>(P, s, sstride, jobs, nft, c.lg); break;
-    case kPml: k_z_update<T, kPml, CLS><<<grid, NT, c.smem, st>>>(P, s, sstride, jobs, nft, c.lg); break;
-    default: k_z_update<T, kRhoForm, CLS><<<grid, NT, c.smem, st>>>(P, s, sstride, jobs, nft, c.lg); break;
+    case kVacuum: launch_ordered(P.order, k_z_update<T, kVacuum, CLS>, grid, NT, c.smem, st, P, s, sstride, jobs, nft, c.lg); break;
+    case kJForm: launch_ordered(P.order, k_z_update<T, kJForm, CLS>, grid, NT, c.smem, st, P, s, sstride, jobs, nft, c.lg); break;
+    case kPml: launch_ordered(P.order, k_z_update<T, kPml, CLS>, grid, NT, c.smem, st, P, s, sstride, jobs, nft, c.lg); break;
+    default: launch_ordered(P.order, k_z_update<T, kRhoForm, CLS>, grid, NT, c.smem, st, P, s, sstride, jobs, nft, c.lg); break;
   }
 }
 

@@ -21,6 +21,7 @@
 
 #include "any_fft.cuh"
 #include "fft_codelets.cuh"
+#include "launch.cuh"
 #include "psatd_internal.h"
 #include "psatd_update.cuh"
 
@@ -50,6 +51,7 @@ __global__ void __launch_bounds__(z_threads<T>(), CLS ? 1 : sizeof(T) == 4 ? 2 :
   cx<T>* g = spec + bx.soff + (int64_t)J.plane * hx + J.m0;
   const int c = threadIdx.x & (tx - 1), i0 = threadIdx.x >> lg, is = blockDim.x >> lg;
   const bool live = c < nm;
+  grid_order(P.order);
   // pass 1 from HBM, lanes over (column, n2); slots >= nft already hold their
   // z spectrum (a cached constant current) and are placed as they are
   if (live) {

@@ -13,6 +13,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "launch.cuh"
 #include "psatd_internal.h"
 
 namespace psatd {
@@ -70,7 +71,7 @@ __device__ __forceinline__ void copy_tile(T* dbase, const T* sbase, const CopyBl
 template <typename T>
 __global__ void __launch_bounds__(256) k_exchange(const BoxDev* __restrict__ dboxes, const BoxDev* __restrict__ sboxes,
                                                   FieldPtrs Dst, FieldPtrs S, const CopyBlk* __restrict__ blocks,
-                                                  const XTile* __restrict__ tiles) {
+                                                  const XTile* __restrict__ tiles, int order) {
   const XTile t = tiles[blockIdx.x];
   const CopyBlk b = blocks[t.blk];
   T* dbase = reinterpret_cast<T*>(Dst.p[blockIdx.y]);
@@ -83,6 +84,7 @@ __global__ void __launch_bounds__(256) k_exchange(const BoxDev* __restrict__ dbo
     sn0 = sb.n[0];
     sn1 = sb.n[1];
   }
+  grid_order(order);
   if (t.vec > 1)
     copy_tile<T, 16 / sizeof(T)>(dbase, sbase, b, t, db, sfoff, sn0, sn1);
   else
@@ -110,6 +112,7 @@ __global__ void __launch_bounds__(256) k_pml_damp(DevPlan P, FieldPtrs F, FieldP
   const int m0 = bx.n[0] - bx.ng_lo[0] - bx.ng_hi[0], m1 = bx.n[1] - bx.ng_lo[1] - bx.ng_hi[1];
   const int m2 = bx.n[2] - bx.ng_lo[2] - bx.ng_hi[2];
   const int64_t cells = (int64_t)m0 * m1 * m2;
+  grid_order(P.order);
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < cells; e += (int64_t)gridDim.x * blockDim.x) {
     const int x = (int)(e % m0), y = (int)((e / m0) % m1), z = (int)(e / ((int64_t)m0 * m1));
     const int g[3] = {pb.origin[0] + x, pb.origin[1] + y, pb.origin[2] + z};
@@ -165,11 +168,12 @@ cudaError_t launch_pml_damp(int prec, const DevPlan& P, const FieldPtrs& f, cons
                             const PmlBox* boxes, int nboxes, const void* tab, const PmlTab& t, cudaStream_t st) {
   for (int b0 = 0; b0 < nboxes; b0 += 65535) {
     dim3 grid(64, (unsigned)std::min(65535, nboxes - b0));
-    if (prec == 32)
-      k_pml_damp<float><<<grid, 256, 0, st>>>(P, f, parts, boxes + b0, (const float*)tab, t);
-    else
-      k_pml_damp<double><<<grid, 256, 0, st>>>(P, f, parts, boxes + b0, (const double*)tab, t);
-    const cudaError_t e = cudaGetLastError();
+    const int order = b0 ? kOrdinary : P.order;
+    const cudaError_t e =
+        prec == 32 ? launch_ordered(order, k_pml_damp<float>, grid, 256, 0, st, P, f, parts, boxes + b0,
+                                    (const float*)tab, t)
+                   : launch_ordered(order, k_pml_damp<double>, grid, 256, 0, st, P, f, parts, boxes + b0,
+                                    (const double*)tab, t);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -178,19 +182,18 @@ cudaError_t launch_pml_damp(int prec, const DevPlan& P, const FieldPtrs& f, cons
 cudaError_t launch_exchange(int prec, const DevPlan& P, const FieldPtrs& f, int nf,
                             const CopyBlk* blocks, const XTile* tiles, int64_t ntiles,
                             cudaStream_t st) {
-  return launch_copy_blocks(prec, P.boxes, P.boxes, f, f, nf, blocks, tiles, ntiles, st);
+  return launch_copy_blocks(prec, P.boxes, P.boxes, f, f, nf, blocks, tiles, ntiles, P.order, st);
 }
 
 cudaError_t launch_copy_blocks(int prec, const BoxDev* dboxes, const BoxDev* sboxes, const FieldPtrs& dst,
                                const FieldPtrs& src, int nf, const CopyBlk* blocks, const XTile* tiles,
-                               int64_t ntiles, cudaStream_t st) {
+                               int64_t ntiles, int order, cudaStream_t st) {
   if (ntiles <= 0 || nf <= 0) return cudaSuccess;
   dim3 grid((unsigned)ntiles, nf);
-  if (prec == 32)
-    k_exchange<float><<<grid, 256, 0, st>>>(dboxes, sboxes, dst, src, blocks, tiles);
-  else
-    k_exchange<double><<<grid, 256, 0, st>>>(dboxes, sboxes, dst, src, blocks, tiles);
-  return cudaGetLastError();
+  return prec == 32
+             ? launch_ordered(order, k_exchange<float>, grid, 256, 0, st, dboxes, sboxes, dst, src, blocks, tiles, order)
+             : launch_ordered(order, k_exchange<double>, grid, 256, 0, st, dboxes, sboxes, dst, src, blocks, tiles,
+                              order);
 }
 
 }  // namespace psatd

@@ -1,0 +1,57 @@
+// Order of a launch against the launch before it in the stream, and the
+// device side of it (programmatic dependent launch).
+//
+//   kOrdinary  starts when everything before it has finished.
+//   kChained   starts while the launch before it drains: its blocks read the
+//              plan's constant tables, then wait for that launch to finish
+//              (grid_order).  For a launch whose predecessor is a single
+//              launch of the same call, so that its end is the end of all work
+//              before it.
+//   kBeside    starts while the launch before it drains and does not wait: for
+//              the second and later launches of one pass over different
+//              boxes, the first of which is kOrdinary.  The launch after the
+//              pass is kOrdinary again.
+//
+// Every kernel here lets its successor start as soon as all its own blocks have
+// (grid_release), so a successor's blocks only take the room that the last
+// wave leaves.
+//
+// Chained are the line kernels (any_lines.cuh, any_z.cuh, the exchange) of calls
+// that launch directly: a PIC cycle of a 64^3 box 71 -> 62 us, forward + inverse
+// FFT of 240 x 200 x 180 187 -> 177 us.  Not the register kernels: a z block that
+// starts on an SM still set up for the plane kernels' shared memory keeps
+// their small L1 (128 boxes of 96^3: 2.90 -> 3.22 ms per step).  Not captured
+// steps: 32^3 FP64 45 -> 56 us per step.  Beside: the register kernels of a batch
+// of many box shapes, 60 launches a step whose tails overlap (40 uneven boxes
+// 1.51 -> 1.27 ms per step).
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "psatd_internal.h"
+
+namespace psatd {
+
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void grid_order(int order) {
+  grid_release();
+  if (order == kChained) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <typename... P, typename... A>
+cudaError_t launch_ordered(int order, void (*kernel)(P...), dim3 grid, int threads, int smem, cudaStream_t st,
+                           A... args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = dim3((unsigned)threads);
+  c.dynamicSmemBytes = (size_t)smem;
+  c.stream = st;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = &attr;
+  c.numAttrs = order == kOrdinary ? 0 : 1;
+  return cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
+
+}  // namespace psatd

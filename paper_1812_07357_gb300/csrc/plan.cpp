@@ -410,6 +410,7 @@ struct psatd_plan {
 
   int64_t field_total = 0;  // elements per field buffer
   int64_t spec_total = 0;   // complex elements per spectrum slot
+  bool chain = false;   // every pass of a step is one launch of a line kernel (kChained in direct launches)
   LineCfg cfg_x, cfg_y, cfg_z, cfg_zonly;   // generic kernels: launches that cover every box
   int smem_pf = 0, smem_pi = 0, smem_zf = 0;
   int buf_pf = 0, buf_pi = 0, rows_pi = 0;     // complex elements per plane buffer
@@ -1097,6 +1098,10 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
     }
   }
   build_gather(P, box_fast, d.flags);
+  {
+    // one launch per pass, each of a line kernel (register z kernels do not wait)
+    P->chain = P->fast_boxes == 0 && P->grp_zreg.empty();
+  }
   // ---- device memory
   CK(P, upload(P, P->hboxes, &P->d_boxes));
   CK(P, upload(P, P->hshapes, &P->d_shapes));
@@ -1641,16 +1646,28 @@ psatd_status psatd_guard_exchange(psatd_plan* P, const psatd_fields* f, const ps
   }
 }
 
+// Orders of the launches of one call (launch.cuh): `chain` (a plan's chain
+// flag, never with per-kernel timing) makes every launch but the call's first
+// kChained; the later launches of a pass over several groups are kBeside the
+// first.  `before`: launches of this call so far.
+static DevPlan in_pass(const psatd_plan* P, const DevPlan& D, bool chain, int64_t before, bool later) {
+  DevPlan d = D;
+  d.order = later && !P->timing ? kBeside : chain && before > 0 ? kChained : kOrdinary;
+  return d;
+}
+
 // S1 along x and y of the field slots fp.p[0..nf) into spectrum slots
 // spec + f * spec_total, on every kernel family; adds the launches.
-static psatd_status forward_xy(psatd_plan* P, const DevPlan& D, const FieldPtrs& fp, int nf, void* spec,
-                               cudaStream_t st, int64_t* launches_out, bool gather = false) {
+static psatd_status forward_xy(psatd_plan* P, const DevPlan& D0, const FieldPtrs& fp, int nf, void* spec,
+                               cudaStream_t st, int64_t* launches_out, bool gather = false, bool chain = false) {
   const int64_t S = P->spec_total;
   int64_t launches = 0;
+  DevPlan D = in_pass(P, D0, chain, *launches_out, false);
   // fast boxes: one plane kernel; generic and pencil boxes: x rows, y columns
   if (!P->grp_pf.empty()) {
     // one launch per register plane shape; the gather tables are indexed by plane_fwd position
     for (const auto& g : P->grp_pf) {
+      D = in_pass(P, D0, chain, *launches_out + launches, &g != &P->grp_pf.front());
       if (g.code < 0) {
         CK(P, timed(P, 0, st, [&] {
              return launch_plane_fwd(P->prec, D, fp, nf, spec, S, P->d_plane_fwd + g.start, g.count, P->buf_pf,
@@ -1675,10 +1692,12 @@ static psatd_status forward_xy(psatd_plan* P, const DevPlan& D, const FieldPtrs&
     ++launches;
   }
   if (P->g_nrows) {
+    D = in_pass(P, D0, chain, *launches_out + launches, false);
     CK(P, timed(P, 0, st, [&] {
          return launch_fwd_x(P->prec, D, fp, nf, spec, S, P->d_rows_all, P->g_nrows, P->cfg_x,
                              gather && !P->ggrid.empty() ? P->d_ggrid : nullptr, fields_out(P->form), st);
        }));
+    D = in_pass(P, D0, chain, *launches_out + launches + 1, false);
     CK(P, timed(P, 1, st, [&] {
          return launch_col(P->prec, -1, 1, D, spec, S, nf, P->d_ycols_all, P->g_nycols, P->cfg_y, st);
        }));
@@ -1739,10 +1758,12 @@ static psatd_status transform_current(psatd_plan* P, const DevPlan& D, const Fie
 
 // S1 (z) + S2 + S3 (z) of one step: every register-z, pencil and generic z
 // pass, on the plan's spectrum workspace.
-static psatd_status z_step(psatd_plan* P, const DevPlan& D, cudaStream_t st, int64_t* launches_out) {
+static psatd_status z_step(psatd_plan* P, const DevPlan& D0, cudaStream_t st, int64_t* launches_out,
+                           bool chain = false) {
   const int NFT = step_slots(P);
   const int64_t S = P->spec_total;
   int64_t launches = 0;
+  DevPlan D = in_pass(P, D0, chain, *launches_out, false);
   const bool one_launch = P->z_one_launch && P->zreg_multi;
   if (one_launch) {
     // every register-z length in one persistent launch, 2 CTAs per SM
@@ -1753,12 +1774,14 @@ static psatd_status z_step(psatd_plan* P, const DevPlan& D, cudaStream_t st, int
     ++launches;
   }
   for (const auto& g : one_launch ? std::vector<psatd_plan::Group>() : P->grp_zreg) {
+    D = in_pass(P, D0, chain, *launches_out + launches, launches > 0);
     CK(P, timed(P, 2, st, [&] {
          return launch_z_reg(P->form, D, P->d_ws, S, P->d_zpen_reg + g.start, g.count, g.code, 0, NFT, P->z_prefetch,
                              st);
        }));
     ++launches;
   }
+  D = in_pass(P, D0, chain, *launches_out + launches, false);
   if (!P->zfast.empty() && P->reg_z) {
     CK(P, timed(P, 2, st, [&] {
          return launch_z_reg(P->form, D, P->d_ws, S, P->d_zfast, (int64_t)P->zfast.size(), P->reg_z, P->reg_zst,
@@ -1788,14 +1811,16 @@ static psatd_status z_step(psatd_plan* P, const DevPlan& D, cudaStream_t st, int
 // damping and the eager guard exchange (with `guards`).  The kernels use the
 // slot index only to offset the field and spectrum pointers, so one slot c
 // alone is inverted by passing its field pointer as slot 0 and its spectrum.
-static psatd_status inverse_step(psatd_plan* P, const DevPlan& D, const FieldPtrs& fp, int nout, void* spec,
-                                 cudaStream_t st, int64_t* launches_out, bool guards) {
+static psatd_status inverse_step(psatd_plan* P, const DevPlan& D0, const FieldPtrs& fp, int nout, void* spec,
+                                 cudaStream_t st, int64_t* launches_out, bool guards, bool chain = false) {
   const int64_t S = P->spec_total;
   int64_t launches = 0;
+  DevPlan D = in_pass(P, D0, chain, *launches_out, false);
   // S3: inverse y+x, interior cells only
   if (!P->grp_pi.empty()) {
     // one launch per register plane shape; the guard segments are indexed by plane_inv position
     for (const auto& g : P->grp_pi) {
+      D = in_pass(P, D0, chain, *launches_out + launches, &g != &P->grp_pi.front());
       if (g.code < 0) {
         CK(P, timed(P, 4, st, [&] {
              return launch_plane_inv(P->prec, D, fp, nout, spec, S, P->d_plane_inv + g.start, g.count, P->buf_pi,
@@ -1821,9 +1846,11 @@ static psatd_status inverse_step(psatd_plan* P, const DevPlan& D, const FieldPtr
     ++launches;
   }
   if (P->g_nrows) {
+    D = in_pass(P, D0, chain, *launches_out + launches, false);
     CK(P, timed(P, 3, st, [&] {
          return launch_col(P->prec, 1, 1, D, spec, S, nout, P->d_g_ycols_int, (int64_t)P->g_ycols_int.size(), P->cfg_y, st);
        }));
+    D = in_pass(P, D0, chain, *launches_out + launches + 1, false);
     CK(P, timed(P, 4, st, [&] {
          return launch_inv_x(P->prec, D, fp, nout, spec, S, P->d_g_rows_int, (int64_t)P->g_rows_int.size(), P->cfg_x, 1, st);
        }));
@@ -1833,6 +1860,7 @@ static psatd_status inverse_step(psatd_plan* P, const DevPlan& D, const FieldPtr
     // absorbing layers, step (2): damp the split parts, rebuild the components
     FieldPtrs parts{};
     for (int q = 0; q < 6; ++q) parts.p[q] = P->pml_parts[q];
+    D = in_pass(P, D0, chain, *launches_out + launches, false);
     CK(P, timed(P, 4, st, [&] {
          return launch_pml_damp(P->prec, D, fp, parts, P->d_pml_boxes, (int)P->pml_boxes.size(), P->d_pml_tab,
                                 P->pml_tab, st);
@@ -1841,6 +1869,7 @@ static psatd_status inverse_step(psatd_plan* P, const DevPlan& D, const FieldPtr
   }
   if (!P->step_tiles.empty() && guards) {
     const int nex = P->form == kPml ? 6 : nout;   // components only, not the increments
+    D = in_pass(P, D0, chain, *launches_out + launches, false);
     CK(P, timed(P, 5, st, [&] {
          return launch_exchange(P->prec, D, fp, nex, P->d_blocks, P->d_step_tiles, (int64_t)P->step_tiles.size(),
                                 st);
@@ -1855,14 +1884,16 @@ static psatd_status inverse_step(psatd_plan* P, const DevPlan& D, const FieldPtr
 // gather: the forward pass reads guard cells from their owners (deferred
 // exchange); guards: the inverse pass stores the guard cells.
 static psatd_status push_step(psatd_plan* P, const DevPlan& D, const FieldPtrs& fp, cudaStream_t st,
-                              int64_t* launches_out, bool gather = false, bool guards = true) {
+                              int64_t* launches_out, bool gather, bool guards, bool in_graph) {
+  const bool chain = P->chain && !P->timing && !in_graph;
+  int64_t n = 0;   // of this step: its first launch is ordinary
   // S1: forward x+y of the slots transformed every step
-  psatd_status r = forward_xy(P, D, fp, step_slots(P), P->d_ws, st, launches_out, gather);
-  if (r != PSATD_OK) return r;
-  r = z_step(P, D, st, launches_out);
-  if (r != PSATD_OK) return r;
+  psatd_status r = forward_xy(P, D, fp, step_slots(P), P->d_ws, st, &n, gather, chain);
+  if (r == PSATD_OK) r = z_step(P, D, st, &n, chain);
   // S3: inverse y+x, interior cells only
-  return inverse_step(P, D, fp, fields_out(P->form), P->d_ws, st, launches_out, guards);
+  if (r == PSATD_OK) r = inverse_step(P, D, fp, fields_out(P->form), P->d_ws, st, &n, guards, chain);
+  *launches_out += n;
+  return r;
 }
 
 // Capture one step of variant v (2 * gather + guards, see push_step) into a
@@ -1899,7 +1930,7 @@ static bool step_graph(psatd_plan* P, const DevPlan& D, const FieldPtrs& fp, int
     return false;
   }
   int64_t n = 0;
-  const psatd_status r = push_step(P, D, fp, P->cap_stream, &n, (v & 2) != 0, (v & 1) != 0);
+  const psatd_status r = push_step(P, D, fp, P->cap_stream, &n, (v & 2) != 0, (v & 1) != 0, true);
   cudaGraph_t g = nullptr;
   const cudaError_t e = cudaStreamEndCapture(P->cap_stream, &g);
   cudaGraphExec_t x = nullptr;
@@ -1943,7 +1974,7 @@ psatd_status psatd_push(psatd_plan* P, const psatd_fields* f, const psatd_source
         CK(P, cudaGraphLaunch(P->graph_exec[v], st));
         launches += P->graph_launches[v];
       } else {
-        r = push_step(P, D, fp, st, &launches, gather, guards);
+        r = push_step(P, D, fp, st, &launches, gather, guards, false);
         if (r != PSATD_OK) return r;
       }
     }
@@ -2177,9 +2208,10 @@ psatd_status psatd_forward_fft(psatd_plan* P, const void* field, void* spectrum,
   fp.p[0] = const_cast<void*>(field);
   cudaStream_t st = (cudaStream_t)stream;
   P->last_stream = st;
-  const DevPlan D = P->dev();
+  DevPlan D = P->dev();
   const int64_t S = P->spec_total;
   CK(P, launch_fwd_x(P->prec, D, fp, 1, spectrum, S, P->d_rows_all, (int64_t)P->rows_all.size(), P->cfg_x, nullptr, 0, st));
+  D.order = kChained;
   CK(P, launch_col(P->prec, -1, 1, D, spectrum, S, 1, P->d_ycols_all, (int64_t)P->ycols_all.size(), P->cfg_y, st));
   CK(P, launch_col(P->prec, -1, 2, D, spectrum, S, 1, P->d_zcols, (int64_t)P->zcols.size(), P->cfg_zonly, st));
   P->last_launches = 3;
@@ -2194,9 +2226,10 @@ psatd_status psatd_inverse_fft(psatd_plan* P, void* spectrum, void* field, void*
   fp.p[0] = field;
   cudaStream_t st = (cudaStream_t)stream;
   P->last_stream = st;
-  const DevPlan D = P->dev();
+  DevPlan D = P->dev();
   const int64_t S = P->spec_total;
   CK(P, launch_col(P->prec, 1, 2, D, spectrum, S, 1, P->d_zcols, (int64_t)P->zcols.size(), P->cfg_zonly, st));
+  D.order = kChained;
   CK(P, launch_col(P->prec, 1, 1, D, spectrum, S, 1, P->d_ycols_all, (int64_t)P->ycols_all.size(), P->cfg_y, st));
   CK(P, launch_inv_x(P->prec, D, fp, 1, spectrum, S, P->d_rows_all, (int64_t)P->rows_all.size(), P->cfg_x, 0, st));
   P->last_launches = 3;
@@ -2570,7 +2603,7 @@ psatd_status psatd_couple(psatd_coupling* c, int32_t direction, void* const* g1_
   const bool to_fft = direction == PSATD_G1_TO_G2;
   CK(P, launch_copy_blocks(P->prec, to_fft ? P->d_boxes : c->d_g1, to_fft ? c->d_g1 : P->d_boxes,
                            to_fft ? f2 : f1, to_fft ? f1 : f2, nfields, c->d_blk[direction], c->d_tiles[direction],
-                           (int64_t)c->tiles[direction].size(), st));
+                           (int64_t)c->tiles[direction].size(), kOrdinary, st));
   P->last_launches = c->tiles[direction].empty() ? 0 : 1;
   return PSATD_OK;
 }

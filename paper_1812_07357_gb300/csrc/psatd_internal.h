@@ -173,6 +173,9 @@ struct alignas(4 * sizeof(T)) Coef4 {
   T x3;   // (sin(theta)/(c K) - dt)/K^2
 };
 
+// Order of a launch against the one before it (launch.cuh).
+enum LaunchOrder { kOrdinary = 0, kChained = 1, kBeside = 2 };
+
 // Device view of a plan, passed by value to every kernel.
 struct DevPlan {
   const BoxDev* boxes;
@@ -182,6 +185,7 @@ struct DevPlan {
   const void* coef;               // Coef4<T>[]
   double c, eps0, dt;
   double cc, ieps, idt, icce;     // c^2, 1/eps0, 1/dt, 1/(c^2 eps0)
+  int32_t order;                  // LaunchOrder of the launch that gets this copy
 };
 
 inline void set_constants(DevPlan& P, double c, double eps0, double dt) {
@@ -192,6 +196,7 @@ inline void set_constants(DevPlan& P, double c, double eps0, double dt) {
   P.ieps = 1.0 / eps0;
   P.idt = 1.0 / dt;
   P.icce = 1.0 / (c * c * eps0);
+  P.order = kOrdinary;
 }
 
 // ---- generic kernels (fft_kernels.cu, any_lines.cuh, any_z.cuh) ---------------------------
@@ -249,7 +254,7 @@ cudaError_t launch_exchange(int prec, const DevPlan& P, const FieldPtrs& f, int 
 // (sboxes, buffers src) may belong to two different layouts.
 cudaError_t launch_copy_blocks(int prec, const BoxDev* dboxes, const BoxDev* sboxes, const FieldPtrs& dst,
                                const FieldPtrs& src, int nf, const CopyBlk* blocks, const XTile* tiles,
-                               int64_t ntiles, cudaStream_t st);
+                               int64_t ntiles, int order, cudaStream_t st);
 // Maximum dynamic shared memory opt-in for all kernels of a precision.
 cudaError_t configure_kernels(int prec, int smem_bytes);
 

@@ -18,6 +18,7 @@
 #include <type_traits>
 
 #include "fft_codelets.cuh"
+#include "launch.cuh"
 #include "psatd_internal.h"
 #include "psatd_update.cuh"
 #include "reg_common.cuh"
@@ -219,6 +220,7 @@ __global__ void __launch_bounds__(z_reg_threads<FORM>(), z_reg_min_blocks<FORM>(
             int pf_dist) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const ColJob J = jobs[blockIdx.x];
+  grid_release();
   // the tile that a CTA launched about pf_dist blocks later will read: fetched
   // into L2 now, so that its loads hit L2 instead of waiting on HBM
   if (pf_dist > 0 && (int)blockIdx.x + pf_dist < njobs)
@@ -368,6 +370,7 @@ __global__ void __launch_bounds__(z_reg4_threads<FORM>(), 2)
              int pf_dist) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const ColJob J = jobs[blockIdx.x];
+  grid_release();
   if (pf_dist > 0 && (int)blockIdx.x + pf_dist < njobs)
     prefetch_z_tile<NZ, FORM, z_reg4_threads<FORM>()>(P, spec, sstride, jobs[blockIdx.x + pf_dist]);
   z_reg4_tile_job<NZ, FORM>(P, spec, sstride, J, nft, smem_raw);
@@ -466,8 +469,8 @@ cudaError_t launch_z_reg(int form, const DevPlan& P, void* spec, int64_t sstride
   dim3 grid((unsigned)njobs);
   const int smem = z_reg_smem(form, n2);
 #define PSATD_ZF(NZV, F, ZS)                                                                      \
-  k_z_reg<NZV, F, ZS><<<grid, z_reg_threads<F>(), smem, st>>>(P, (float2*)spec, sstride, jobs, nft, \
-                                                               (int)njobs, pf_dist)
+  launch_ordered(P.order, k_z_reg<NZV, F, ZS>, grid, z_reg_threads<F>(), smem, st, P, (float2*)spec, \
+                 sstride, jobs, nft, (int)njobs, pf_dist)
 #define PSATD_ZL(NZV)                                                    \
   if (n2 == NZV) {                                                      \
     if (form == kVacuum) {                                              \
@@ -493,14 +496,14 @@ cudaError_t launch_z_reg(int form, const DevPlan& P, void* spec, int64_t sstride
 #define PSATD_ZL(NZV)                                                                                     \
   if (n2 == NZV) {                                                                                       \
     if (form == kVacuum)                                                                                 \
-      k_z_reg4<NZV, kVacuum><<<grid, z_reg4_threads<kVacuum>(), smem, st>>>(P, (float2*)spec, sstride, jobs, \
-                                                                            nft, (int)njobs, pf_dist);    \
+      launch_ordered(P.order, k_z_reg4<NZV, kVacuum>, grid, z_reg4_threads<kVacuum>(), smem, st, P, (float2*)spec,  \
+                     sstride, jobs, nft, (int)njobs, pf_dist);    \
     else if (form == kJForm)                                                                             \
-      k_z_reg4<NZV, kJForm><<<grid, z_reg4_threads<kJForm>(), smem, st>>>(P, (float2*)spec, sstride, jobs,   \
-                                                                          nft, (int)njobs, pf_dist);      \
+      launch_ordered(P.order, k_z_reg4<NZV, kJForm>, grid, z_reg4_threads<kJForm>(), smem, st, P, (float2*)spec,  \
+                     sstride, jobs, nft, (int)njobs, pf_dist);      \
     else                                                                                                 \
-      k_z_reg4<NZV, kRhoForm><<<grid, z_reg4_threads<kRhoForm>(), smem, st>>>(P, (float2*)spec, sstride,     \
-                                                                              jobs, nft, (int)njobs, pf_dist); \
+      launch_ordered(P.order, k_z_reg4<NZV, kRhoForm>, grid, z_reg4_threads<kRhoForm>(), smem, st, P, (float2*)spec,  \
+                     sstride, jobs, nft, (int)njobs, pf_dist);                                            \
   }
   PSATD_REG_Z4(PSATD_ZL)
 #undef PSATD_ZL

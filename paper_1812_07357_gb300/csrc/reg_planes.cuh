@@ -24,6 +24,7 @@
 #pragma once
 #include <cooperative_groups.h>
 
+#include "launch.cuh"
 #include "reg_common.cuh"
 
 namespace psatd {
@@ -152,6 +153,7 @@ __global__ void __launch_bounds__(reg_plane_threads<L, NY>(), reg_plane_min_bloc
   const int2 J = jobs[blockIdx.x];
   const int f = blockIdx.y;
   const BoxDev bx = P.boxes[J.x];
+  grid_release();
   plane_load<N0, NY, NT>(P, F, buf, J, f, bx, gstart, gsegs, ggrid, ngather);
   // x: row r -> half spectrum X[0..L] written back into the same row
   if (threadIdx.x < NY) {
@@ -277,6 +279,7 @@ __global__ void __launch_bounds__(reg_plane_threads<L, NY>(), reg_plane_min_bloc
   const int2 J = jobs[blockIdx.x];
   const int f = blockIdx.y;
   const BoxDev bx = P.boxes[J.x];
+  grid_release();
   const int ylo = bx.ng_lo[1], yhi = NY - bx.ng_hi[1], ni = yhi - ylo;
   const int xlo = bx.ng_lo[0], nxi = N0 - bx.ng_lo[0] - bx.ng_hi[0];
   const float2* g = spec + f * sstride + bx.soff + (int64_t)J.y * NY * HX;
@@ -422,6 +425,7 @@ __global__ void __launch_bounds__(wide_threads<L, NY>(), wide_min_blocks<L, NY>(
   const int2 J = jobs[blockIdx.x];
   const int f = blockIdx.y;
   const BoxDev bx = P.boxes[J.x];
+  grid_release();
   plane_load<N0, NY, NT>(P, F, buf, J, f, bx, gstart, gsegs, ggrid, ngather);
   const int t = threadIdx.x;
   // x, stage 1: thread (row r, q): DFT of the packed samples z[q + GX j]
@@ -567,6 +571,7 @@ __global__ void __launch_bounds__(wide_threads<L, NY>(), wide_min_blocks<L, NY>(
   const int2 J = jobs[blockIdx.x];
   const int f = blockIdx.y;
   const BoxDev bx = P.boxes[J.x];
+  grid_release();
   const int ylo = bx.ng_lo[1], yhi = NY - bx.ng_hi[1], ni = yhi - ylo;
   const int xlo = bx.ng_lo[0], nxi = N0 - bx.ng_lo[0] - bx.ng_hi[0];
   {
@@ -821,6 +826,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split_threads<L, NY>
   const int2 J = jobs[pj];
   const int f = blockIdx.y;
   const BoxDev bx = P.boxes[J.x];
+  grid_release();
   plane_load_rows<N0, NY, NT, NH>(F, buf, J, f, bx, pj, h * NH, gstart, gsegs, ggrid, ngather);
   const int t = threadIdx.x;
   // x, stage 1 on the CTA's rows (as k_plane_fwd_wide)
@@ -968,14 +974,14 @@ bool plane_fwd_shape(int code, dim3 grid, const DevPlan& P, const FieldPtrs& f, 
   if constexpr (PART == PSATD_PLANE_PART) {
     if (code != CODE) return false;
     if constexpr (plane_is_split<L, NY>())
-      k_plane_fwd_split<L, NY><<<dim3(2 * grid.x, grid.y), split_threads<L, NY>(), split_smem<L, NY>(), st>>>(
-          P, f, (float2*)spec, sstride, jobs, gstart, gsegs, ggrid, ngather);
+      launch_ordered(P.order, k_plane_fwd_split<L, NY>, dim3(2 * grid.x, grid.y), split_threads<L, NY>(), split_smem<L, NY>(),
+                     st, P, f, (float2*)spec, sstride, jobs, gstart, gsegs, ggrid, ngather);
     else if constexpr (plane_is_wide<L, NY>())
-      k_plane_fwd_wide<L, NY><<<grid, wide_threads<L, NY>(), plane_fwd_bytes<L, NY>(), st>>>(
-          P, f, (float2*)spec, sstride, jobs, gstart, gsegs, ggrid, ngather);
+      launch_ordered(P.order, k_plane_fwd_wide<L, NY>, grid, wide_threads<L, NY>(), plane_fwd_bytes<L, NY>(),
+                     st, P, f, (float2*)spec, sstride, jobs, gstart, gsegs, ggrid, ngather);
     else
-      k_plane_fwd_reg<L, NY><<<grid, reg_plane_threads<L, NY>(), plane_fwd_bytes<L, NY>(), st>>>(
-          P, f, (float2*)spec, sstride, jobs, gstart, gsegs, ggrid, ngather);
+      launch_ordered(P.order, k_plane_fwd_reg<L, NY>, grid, reg_plane_threads<L, NY>(), plane_fwd_bytes<L, NY>(),
+                     st, P, f, (float2*)spec, sstride, jobs, gstart, gsegs, ggrid, ngather);
     return true;
   } else {
     return false;
@@ -988,11 +994,11 @@ bool plane_inv_shape(int code, dim3 grid, const DevPlan& P, const FieldPtrs& f, 
   if constexpr (PART == PSATD_PLANE_PART) {
     if (code != CODE) return false;
     if constexpr (plane_is_wide<L, NY>())
-      k_plane_inv_wide<L, NY><<<grid, wide_threads<L, NY>(), plane_inv_bytes<L, NY>(), st>>>(
-          P, f, (const float2*)spec, sstride, jobs, seg_start, segs);
+      launch_ordered(P.order, k_plane_inv_wide<L, NY>, grid, wide_threads<L, NY>(), plane_inv_bytes<L, NY>(),
+                     st, P, f, (const float2*)spec, sstride, jobs, seg_start, segs);
     else
-      k_plane_inv_reg<L, NY><<<grid, reg_plane_threads<L, NY>(), plane_inv_bytes<L, NY>(), st>>>(
-          P, f, (const float2*)spec, sstride, jobs, seg_start, segs);
+      launch_ordered(P.order, k_plane_inv_reg<L, NY>, grid, reg_plane_threads<L, NY>(), plane_inv_bytes<L, NY>(),
+                     st, P, f, (const float2*)spec, sstride, jobs, seg_start, segs);
     return true;
   } else {
     return false;
