@@ -133,7 +133,8 @@ typedef struct {
  * position.  Requirements: PSATD_VACUUM (no current in the layers), not
  * PSATD_NODAL, not PSATD_DECOMP_INDEPENDENT, 0 <= width[d] <= global_n[d]/2,
  * sigma_max[d] >= 0, 0 <= order <= 16; the plan then runs the generic
- * kernels and stores the guards every step.  The plan owns one stored split
+ * kernels (x and y passes of FP32 boxes with a register plane shape on those)
+ * and stores the guards every step.  The plan owns one stored split
  * part per component (E_xy, E_yz, E_zx, B_xy, B_yz, B_zx; the other part is
  * the component minus it), zero at creation: start with fields that vanish
  * inside the layers, or set the parts through psatd_plan_pml_part. */

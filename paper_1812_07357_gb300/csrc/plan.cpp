@@ -832,9 +832,13 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
   // kernels and a z-pass kernel for its z length (register z, shared-memory
   // plane z or pencil z)
   auto reg_code_of = [&](const psatd_box& b, const ShapeDev& sh) {
-    if (P->prec != 32 || (d.flags & PSATD_GENERIC_KERNELS) || P->form == kPml) return -1;
+    if (P->prec != 32 || (d.flags & PSATD_GENERIC_KERNELS)) return -1;
     const int c = reg_shape_code(sh.L, b.n[1]);
     if (c < 0 || reg_fwd_smem(c) > optin || reg_inv_smem(c) > optin) return -1;
+    if (P->form == kPml) {   // absorbing layers: the generic z pass takes any z length
+      P->reg_planes_used = true;
+      return P->reg_planes ? c : -1;
+    }
     const int n2 = b.n[2], szf = z_fast_smem(P->prec, P->form, n2);
     const bool zr = z_reg_ok(n2) && z_reg_smem(P->form, n2) <= optin;
     const bool zf = sh.fz >= 0 && szf <= optin;
@@ -890,7 +894,9 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
       // z pass: the shared-memory plane z kernel (or the register z kernel,
       // chosen below) where the z length has one, else the generic z pass
       // (or its own register z kernel)
-      if (sh.fz >= 0 && sm_zf <= optin) {
+      if (P->form == kPml) {
+        z_boxes(bi, false);
+      } else if (sh.fz >= 0 && sm_zf <= optin) {
         for (int y = 0; y < n1; ++y)
           for (int m = 0; m < L; m += tile) P->zfast.push_back({bi, y, m, std::min(tile, L - m)});
         // the Nyquist column mx = L in tiles of consecutive y (negative count)
@@ -1046,10 +1052,12 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
   // blocks whose source box runs on the generic kernels.  Blocks outside a
   // non-periodic domain (zero fill) keep the value written by the explicit
   // psatd_guard_exchange: no step writes those cells.
+  // With absorbing layers the step's exchange follows the damping, so nothing
+  // is fused.
   std::vector<char> box_fast(P->boxes.size(), 0);
   std::map<std::pair<int, int>, int> plane_index;  // (box, z) -> plane_inv index
   for (int i = 0; i < (int)P->plane_inv.size(); ++i) {
-    box_fast[P->plane_inv[i].x] = 1;
+    box_fast[P->plane_inv[i].x] = P->form != kPml;
     plane_index[{P->plane_inv[i].x, P->plane_inv[i].y}] = i;
   }
   std::vector<std::vector<GuardSeg>> per_plane(P->plane_inv.size());

@@ -122,3 +122,35 @@ def test_layers_at_tile_edges(prec, n):
     for k in O.SPLIT:
         err = np.linalg.norm(parts[k][0] - ref[k][0])
         assert err <= {64: 1e-12, 32: 2e-5}[prec] * np.linalg.norm(ref[k][0]), k
+
+
+@pytest.mark.parametrize("n1", [48, 60])
+def test_layers_on_register_planes(n1):
+    """FP32 boxes of a register plane shape: x and y on the plane kernels, z on
+    the generic pass (lengths with and without a register z kernel), layers on
+    the faces of an open domain, the exchange after the damping."""
+    from paper_1812_07357_gb300.solver import Plan
+    lay = I.local_layout((80, 2 * n1 - 24, 36), (2, 2, 2), (4, 6, 3), 8, periodic=(0, 0, 1))
+    rng = np.random.default_rng(47)
+    fields = {}
+    for k in O.COMPS:
+        g = rng.standard_normal(lay.global_n[::-1])
+        fields[k] = I.round_to(I.scatter_global(g, lay), np.float32)
+    pml = dict(width=(4, 3, 2), sigma_max=(0.5, 0.4, 0.3), order=2)
+    plan = Plan(lay, (1.0,) * 3, 0.7, precision=32, sources="vacuum", pml=pml)
+    assert plan.fast_boxes == 8 and not plan.deferred_exchange
+    df = plan.pack_fields(fields)
+    plan.push(df, None, 3)
+    plan.sync()
+    got = plan.unpack_fields(df)
+    parts = {k: plan.unpack(v) for k, v in plan.pml_parts().items()}
+    plan.close()
+    ref = O.push(lay, fields, {}, 3, (1.0,) * 3, 0.7, pml=pml)
+    assert_fields(lay, got, ref, O.COMPS, 32)
+    for k in O.COMPS:   # guards stored after the damping
+        for g, r in zip(got[k], ref[k]):
+            assert np.abs(g - r).max() <= 2e-4 * np.abs(r).max(), k
+    for k in O.SPLIT:
+        num = sum(np.linalg.norm((a - b)[3:-3, 6:-6, 4:-4]) ** 2 for a, b in zip(parts[k], ref[k])) ** 0.5
+        den = sum(np.linalg.norm(b[3:-3, 6:-6, 4:-4]) ** 2 for b in ref[k]) ** 0.5
+        assert num <= 2e-5 * den, k
