@@ -87,15 +87,20 @@ void line_cover(LineCfg& c, int prec, const AxisPlan& a, bool rows) {
 
 // Columns per z tile (a power of two, its logarithm in c.lg) and the shared
 // memory of the longest line n2_max: the widest tile of at most 128-byte rows
-// that leaves room for three blocks per SM and gives the `columns` columns of
-// the launch a tile per SM (64^3, 10 slots: 264 tiles of 8 columns run at once,
-// 528 of 4 columns took two waves, 16.5 us against 12); `widest` > 0: no wider than that.
+// that leaves room for the blocks an SM can hold (FP32 two of 256 threads: two
+// boxes of 384 x 256 x 256 2.90 ms per step with 8 columns, 98 KB, against 3.26
+// with 4; FP64 three of 128: 128^3 rho form 2.62 ms either way, 64 x 64 x 256
+// 0.93 against 0.98 with two wider ones) and gives the `columns` columns of the
+// launch a tile per SM (64^3, 10 slots: 264 tiles of 8 columns run at once, 528
+// of 4 columns took two waves, 16.5 us against 12); `widest` > 0: no wider than
+// that.
 void z_cover(LineCfg& c, int prec, int form, int n2_max, int64_t columns, int widest, int sms, int optin) {
   const int csz = prec == 32 ? 8 : 16, ns = spec_slots(form);
   const int lo = prec == 32 ? 2 : 1, hi = prec == 32 ? 4 : 3;   // log2 of the narrowest and widest tile
+  const int budget = (prec == 32 ? 112 : 75) * 1024;
   auto bytes = [&](int lg) { return ns * z_slot_pitch(csz, n2_max, 1 << lg) * csz; };
   int lg = hi;
-  while (lg > lo && (bytes(lg) > 75 * 1024 || (columns >> lg) < sms)) --lg;
+  while (lg > lo && (bytes(lg) > budget || (columns >> lg) < sms)) --lg;
   while (lg > lo - 1 && (bytes(lg) > optin || (widest > 0 && (1 << lg) > widest))) --lg;
   c.lg = lg;
   c.smem = bytes(lg);
