@@ -66,11 +66,26 @@ __global__ void __launch_bounds__(z_threads<T>(), CLS ? 1 : sizeof(T) == 4 ? 2 :
             [&](int k, int, cx<T> v) { b[(k * l.r2 + n2i) << lg] = v; });
       }
     });
-    for (int s = nft; s < FIN; ++s)
-      for (int p = i0; p < n2; p += is) {
-        const int k1 = line_div(p, mr);
-        sm[s * SP + (p << lg) + c] = g[s * sstride + (int64_t)l.freq(k1, p - k1 * l.r2) * zst + c];
-      }
+    if constexpr (FIN > fields_in(kVacuum)) {
+      constexpr int U = 4, NJ = 3;   // a current has three slots; 12 loads before any is stored
+      if (nft + NJ == FIN)
+        for (int p0 = i0; p0 < n2; p0 += U * is) {
+          cx<T> v[U][NJ];
+#pragma unroll
+          for (int i = 0; i < U; ++i) {
+            const int p = p0 + i * is, k1 = line_div(p, mr);
+            const cx<T>* src = g + nft * sstride + (int64_t)l.freq(k1, p - k1 * l.r2) * zst + c;
+#pragma unroll
+            for (int q = 0; q < NJ; ++q)
+              if (p < n2) v[i][q] = src[q * sstride];
+          }
+#pragma unroll
+          for (int i = 0; i < U; ++i)
+#pragma unroll
+            for (int q = 0; q < NJ; ++q)
+              if (p0 + i * is < n2) sm[(nft + q) * SP + ((p0 + i * is) << lg) + c] = v[i][q];
+        }
+    }
   }
   __syncthreads();
   // pass 2 in place, lanes over (column, slot)

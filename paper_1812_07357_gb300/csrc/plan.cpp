@@ -827,23 +827,12 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
            L <= fast_max_x(P->prec) && sm_pf <= optin && sm_pi <= optin &&
            z_fast_smem(P->prec, P->form, n2) <= optin;
   };
-  // register plane shape of a box, or -1
-  // register plane shape of a box, or -1: a shape with register plane
-  // kernels and a z-pass kernel for its z length (register z, shared-memory
-  // plane z or pencil z)
+  // register plane shape of a box, or -1 (its z pass: a register z kernel, the
+  // shared-memory plane z kernel or the generic one, which takes any length)
   auto reg_code_of = [&](const psatd_box& b, const ShapeDev& sh) {
     if (P->prec != 32 || (d.flags & PSATD_GENERIC_KERNELS)) return -1;
     const int c = reg_shape_code(sh.L, b.n[1]);
     if (c < 0 || reg_fwd_smem(c) > optin || reg_inv_smem(c) > optin) return -1;
-    if (P->form == kPml) {   // absorbing layers: the generic z pass takes any z length
-      P->reg_planes_used = true;
-      return P->reg_planes ? c : -1;
-    }
-    const int n2 = b.n[2], szf = z_fast_smem(P->prec, P->form, n2);
-    const bool zr = z_reg_ok(n2) && z_reg_smem(P->form, n2) <= optin;
-    const bool zf = sh.fz >= 0 && szf <= optin;
-    const bool zp = sh.pz >= 0 && n2 <= pencil_max_z(P->prec) && szf <= optin;
-    if (!(zr || zf || zp)) return -1;
     P->reg_planes_used = true;
     return P->reg_planes ? c : -1;
   };
@@ -854,7 +843,7 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
   auto z_boxes = [&](int bi, bool family) {
     const psatd_box& b = P->boxes[bi];
     if (P->prec == 32 && family) P->pen_reg_z_used = true;
-    if (P->prec == 32 && family && P->pen_reg_z && z_reg_ok(b.n[2]) && z_reg_smem(P->form, b.n[2]) <= optin &&
+    if (P->prec == 32 && family && P->pen_reg_z && z_reg_ok(P->form, b.n[2]) && z_reg_smem(P->form, b.n[2]) <= optin &&
         z_reg_multi_smem(P->form) <= optin) {
       const int L = b.n[0] / 2, n1 = b.n[1], rt = z_reg_tile_width(P->form, b.n[2]);
       for (int y = 0; y < n1; ++y)
@@ -896,6 +885,8 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
       // (or its own register z kernel)
       if (P->form == kPml) {
         z_boxes(bi, false);
+      } else if (P->prec == 32 && z_reg_yields(P->form, n2)) {
+        z_boxes(bi, true);
       } else if (sh.fz >= 0 && sm_zf <= optin) {
         for (int y = 0; y < n1; ++y)
           for (int m = 0; m < L; m += tile) P->zfast.push_back({bi, y, m, std::min(tile, L - m)});
@@ -985,7 +976,7 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
     }
     const bool zreg_all = std::all_of(P->zfast.begin(), P->zfast.end(), [&](const ColJob& j) {
       const int n2 = P->boxes[j.box].n[2];
-      return z_reg_ok(n2) && z_reg_smem(P->form, n2) <= optin && z_reg_multi_smem(P->form) <= optin;
+      return z_reg_ok(P->form, n2) && z_reg_smem(P->form, n2) <= optin && z_reg_multi_smem(P->form) <= optin;
     });
     if (nz == -1 && all_reg && zreg_all) P->pen_reg_z_used = true;
     if (nz == -1 && all_reg && zreg_all && P->pen_reg_z) {
@@ -1003,9 +994,11 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
     }
   }
   group(P->zpen_reg, [&](const ColJob& j) { return P->boxes[j.box].n[2]; }, P->grp_zreg);
-  P->zreg_multi = !P->zpen_reg.empty() && std::all_of(P->grp_zreg.begin(), P->grp_zreg.end(), [](const auto& g) {
-    return z_reg_multi_ok(g.code) != 0;
-  });
+  P->zreg_multi = !P->zpen_reg.empty() &&
+                  std::all_of(P->grp_zreg.begin(), P->grp_zreg.end(),
+                              [](const auto& g) { return z_reg_multi_ok(g.code) != 0; }) &&
+                  std::none_of(zgen.begin(), zgen.end(),
+                               [&](int bi) { return z_reg_yields(P->form, P->boxes[bi].n[2]) != 0; });
   if (P->fast_boxes && P->prec == 32 && !P->zfast.empty()) {
     // one register z length for every fast box, or none
     int nz = -2;
@@ -1014,7 +1007,7 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
       nz = (nz == -2 || nz == n2) ? n2 : -1;
       if (nz == -1) break;
     }
-    if (nz > 0 && z_reg_ok(nz) && z_reg_smem(P->form, nz) <= optin) P->reg_z = nz;
+    if (nz > 0 && z_reg_ok(P->form, nz) && z_reg_smem(P->form, nz) <= optin) P->reg_z = nz;
     // the z stride, when every fast box shares it
     for (const ColJob& j : P->zfast) {
       const int zs = P->boxes[j.box].n[1] * (P->boxes[j.box].n[0] / 2 + 1);

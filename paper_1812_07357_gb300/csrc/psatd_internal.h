@@ -309,8 +309,10 @@ PSATD_DECLARE_PLANE_PART(plane_part2)
 PSATD_DECLARE_PLANE_PART(plane_part3)
 #undef PSATD_DECLARE_PLANE_PART
 // register z kernel (FP32, tiles of z_reg_tile_width(form, n2) columns) for z
-// length n2 (thread pairs per column; thread quads for 128 and 192)
-int z_reg_ok(int n2);
+// length n2 (thread pairs per column; thread quads for 128 and 192, vacuum form)
+int z_reg_ok(int form, int n2);
+// a quad length of a form with sources, for which the generic z pass is faster
+int z_reg_yields(int form, int n2);
 int z_reg_multi_ok(int n2);   // a length the persistent multi-length kernel takes
 int z_reg_smem(int form, int n2);
 int z_reg_tile_width(int form, int n2);

@@ -269,9 +269,11 @@ __global__ void __launch_bounds__(z_reg_threads<FORM>(), z_reg_min_blocks<FORM>(
 // the half-length spectrum of their half (rows of the pair kernel's layout),
 // the update stage is the pair kernel's, and the inverse mirrors the forward
 // (split by shuffles, length-NZ/4 inverse DFTs, interior z planes stored).
+// The vacuum form only: with 9 or 10 slots its tiles have 4 columns, and the
+// generic z pass (8 columns) is faster (8 boxes of 192^3: J form 4.48 -> 4.04 ms
+// per step, rho form 4.99 -> 4.71; vacuum 2.93 against 3.00).
 #define PSATD_REG_Z4(X) X(128) X(192)
-// columns per tile: 8 (the 6-slot vacuum form), 4 with sources
-constexpr int z_reg4_tile(int form) { return form == kVacuum ? 8 : 4; }
+constexpr int z_reg4_tile(int) { return 8; }   // columns per tile
 template <int FORM>
 constexpr int z_reg4_threads() {
   return (4 * fields_in(FORM) * z_reg4_tile(FORM) + 31) / 32 * 32;
@@ -425,13 +427,12 @@ static bool z_reg_quad(int n2) {
   return false;
 }
 
-int z_reg_ok(int n2) {
-#define PSATD_ZC(NZV) \
-  if (n2 == NZV) return 1;
-  PSATD_REG_Z(PSATD_ZC)
-#undef PSATD_ZC
-  return z_reg_quad(n2) ? 1 : 0;
+int z_reg_ok(int form, int n2) {
+  if (z_reg_multi_ok(n2)) return 1;
+  return z_reg_quad(n2) && form == kVacuum ? 1 : 0;
 }
+
+int z_reg_yields(int form, int n2) { return z_reg_quad(n2) && form != kVacuum ? 1 : 0; }
 
 int z_reg_multi_ok(int n2) {
 #define PSATD_ZC(NZV) \
@@ -495,15 +496,9 @@ cudaError_t launch_z_reg(int form, const DevPlan& P, void* spec, int64_t sstride
 #undef PSATD_ZF
 #define PSATD_ZL(NZV)                                                                                     \
   if (n2 == NZV) {                                                                                       \
-    if (form == kVacuum)                                                                                 \
-      launch_ordered(P.order, k_z_reg4<NZV, kVacuum>, grid, z_reg4_threads<kVacuum>(), smem, st, P, (float2*)spec,  \
-                     sstride, jobs, nft, (int)njobs, pf_dist);    \
-    else if (form == kJForm)                                                                             \
-      launch_ordered(P.order, k_z_reg4<NZV, kJForm>, grid, z_reg4_threads<kJForm>(), smem, st, P, (float2*)spec,  \
-                     sstride, jobs, nft, (int)njobs, pf_dist);      \
-    else                                                                                                 \
-      launch_ordered(P.order, k_z_reg4<NZV, kRhoForm>, grid, z_reg4_threads<kRhoForm>(), smem, st, P, (float2*)spec,  \
-                     sstride, jobs, nft, (int)njobs, pf_dist);                                            \
+    if (form != kVacuum) return cudaErrorInvalidValue;                                                    \
+    launch_ordered(P.order, k_z_reg4<NZV, kVacuum>, grid, z_reg4_threads<kVacuum>(), smem, st, P, (float2*)spec,  \
+                   sstride, jobs, nft, (int)njobs, pf_dist);                                              \
   }
   PSATD_REG_Z4(PSATD_ZL)
 #undef PSATD_ZL
@@ -628,7 +623,7 @@ cudaError_t configure_reg_kernels(int smem) {
         cudaFuncSetAttribute(k_z_reg4<NZV, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, z_reg_smem(F, NZV)); \
     if (r != cudaSuccess) e = r;                                                                          \
   }
-#define PSATD_ZS(NZV) PSATD_ZA(NZV, kVacuum) PSATD_ZA(NZV, kJForm) PSATD_ZA(NZV, kRhoForm)
+#define PSATD_ZS(NZV) PSATD_ZA(NZV, kVacuum)
   PSATD_REG_Z4(PSATD_ZS)
 #undef PSATD_ZS
 #undef PSATD_ZA
