@@ -34,10 +34,13 @@
 namespace psatd {
 namespace {
 
-// Lines of a tile: 128 bytes of adjacent complex columns, or as many rows.
+// Lines of a tile (adjacent complex columns, or rows), a power of two 1 << lg:
+// FP32 16, 128 bytes of columns; FP64 8 or 16, whichever wastes fewer lanes
+// (line_lg: an FP64 instruction costs a warp the same however few lanes it has).
+constexpr int kMaxLines = 16;
 template <typename T>
-__host__ __device__ constexpr int line_tile() {
-  return 128 / (2 * (int)sizeof(T));
+__device__ __forceinline__ int line_lg(int lg) {
+  return sizeof(T) == 4 ? 4 : lg;
 }
 
 // Row pitch of the FP32 x kernels in shared memory: sub-transform k1 at
@@ -54,10 +57,10 @@ __host__ __device__ constexpr int z_slot_pitch(int csz, int n2, int tx) {
 }
 
 // Threads of a block at most: a tile times the largest radix of the class
-// (class 0: radices up to 16, class 1: up to 32).
+// (class 0: radices up to 16, class 1: up to 32; FP64 class 1 in tiles of 8).
 template <typename T, int CLS>
 constexpr int line_threads() {
-  return line_tile<T>() * (CLS ? 32 : 16);
+  return sizeof(T) == 8 && CLS ? 8 * 32 : kMaxLines * (CLS ? 32 : 16);
 }
 
 // Call f(std::integral_constant<int, r>) for a run-time radix r.

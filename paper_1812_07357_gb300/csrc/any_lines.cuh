@@ -128,8 +128,8 @@ __device__ __forceinline__ void split_rows(const cx<T>* sm, int pitch, int nr, i
 // them, up to three bands of columns per row from the plane's gather grid.
 template <typename T>
 struct RowBands {
-  int64_t src[line_tile<T>()][3];   // element x of band i is src[.][i] + x
-  int x[line_tile<T>()][2];         // the bands' first columns (past the first band)
+  int64_t src[kMaxLines][3];   // element x of band i is src[.][i] + x
+  int x[kMaxLines][2];         // the bands' first columns (past the first band)
   __device__ __forceinline__ int64_t at(int r, int col) const {
     return src[r][(col >= x[r][0]) + (col >= x[r][1])] + col;
   }
@@ -138,10 +138,10 @@ struct RowBands {
 template <typename T, int CLS, bool GATHER>
 __global__ void __launch_bounds__(line_threads<T, CLS>())
     k_fwd_x(DevPlan P, FieldPtrs F, cx<T>* spec, int64_t sstride, const RowJob* __restrict__ jobs,
-            const GatherGrid* __restrict__ ggrid, int ngather) {
+            const GatherGrid* __restrict__ ggrid, int ngather, int lg) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<T>* sm = reinterpret_cast<cx<T>*>(smem_raw);
-  constexpr int W = line_tile<T>();
+  const int lw = line_lg<T>(lg), W = 1 << lw;
   const RowJob J = jobs[blockIdx.x];
   const int f = blockIdx.y;
   const BoxDev& bx = P.boxes[J.box];
@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(line_threads<T, CLS>())
     }
     cp_async_wait();
     __syncthreads();
-    const int c = threadIdx.x % W, g = threadIdx.x / W;
+    const int c = threadIdx.x & (W - 1), g = threadIdx.x >> lw;
     const bool live = c < J.nr;
     rows_pass1<T, -1, CLS>(sm + c * PX, l, g, live, tw);
     rows_pass2<T, -1, CLS>(sm + c * PX, l, g, live);
@@ -227,16 +227,16 @@ __global__ void __launch_bounds__(line_threads<T, CLS>())
 // ---------------------------------------------------------------------------
 template <typename T, int DIR, int CLS>
 __global__ void __launch_bounds__(line_threads<T, CLS>()) k_col(DevPlan P, cx<T>* spec, int64_t sstride, int axis,
-                                                                const ColJob* __restrict__ jobs) {
+                                                                const ColJob* __restrict__ jobs, int lg) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr int W = line_tile<T>();
+  const int lw = line_lg<T>(lg), W = 1 << lw;
   const ColJob J = jobs[blockIdx.x];
   const BoxDev& bx = P.boxes[J.box];
   const ShapeDev& sh = P.shapes[bx.shape];
   const int hx = sh.hx, n1 = bx.n[1];
   const Line l(axis == 1 ? sh.ay : sh.az);
   const cx<T>* tw = cpool<T>(P) + (axis == 1 ? sh.ay.tw : sh.az.tw);
-  const int c = threadIdx.x % W, g0 = threadIdx.x / W, gs = blockDim.x / W;
+  const int c = threadIdx.x & (W - 1), g0 = threadIdx.x >> lw, gs = blockDim.x >> lw;
   const bool live = c < J.nm;
   // first element of this lane's column, and the step between its samples
   int m = J.m0 + c, pl = J.plane;
@@ -249,14 +249,14 @@ __global__ void __launch_bounds__(line_threads<T, CLS>()) k_col(DevPlan P, cx<T>
     stride = hx;
   }
   cx<T>* g = spec + blockIdx.y * sstride + bx.soff + (int64_t)pl * (axis == 1 ? n1 * hx : hx) + m;
-  cx<T>* col = reinterpret_cast<cx<T>*>(smem_raw) + c;   // place p of the column at col[p * W]
+  cx<T>* col = reinterpret_cast<cx<T>*>(smem_raw) + c;   // place p of the column at col[p << lw]
   grid_order(P.order);
   if (live)
     with_radix<CLS>(l.r1, [&](auto rc) {
       for (int n2 = g0; n2 < l.r2; n2 += gs)
         line_pass1<T, decltype(rc)::value, DIR, true>(
             l, n2, tw, [&](int i) { return g[(int64_t)i * stride]; },
-            [&](int k, int, cx<T> v) { col[(k * l.r2 + n2) * W] = v; });
+            [&](int k, int, cx<T> v) { col[(k * l.r2 + n2) << lw] = v; });
     });
   __syncthreads();
   if (live)
@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(line_threads<T, CLS>()) k_col(DevPlan P, cx<T>
       for (int k1 = g0; k1 < l.r1; k1 += gs) {
         cx<T> v[R];
 #pragma unroll
-        for (int j = 0; j < R; ++j) v[j] = col[(k1 * R + j) * W];
+        for (int j = 0; j < R; ++j) v[j] = col[(k1 * R + j) << lw];
         Dft<T, R, DIR>::run(v);
         int k = l.out0(k1);
 #pragma unroll
@@ -286,10 +286,10 @@ __global__ void __launch_bounds__(line_threads<T, CLS>()) k_col(DevPlan P, cx<T>
 template <typename T, int CLS>
 __global__ void __launch_bounds__(line_threads<T, CLS>(), sizeof(T) == 4 && !CLS ? 3 : 1) k_inv_x(DevPlan P, FieldPtrs F, const cx<T>* spec,
                                                                   int64_t sstride, const RowJob* __restrict__ jobs,
-                                                                  int interior_only) {
+                                                                  int interior_only, int lg) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<T>* sm = reinterpret_cast<cx<T>*>(smem_raw);
-  constexpr int W = line_tile<T>();
+  const int lw = line_lg<T>(lg), W = 1 << lw;
   const RowJob J = jobs[blockIdx.x];
   const int f = blockIdx.y;
   const BoxDev& bx = P.boxes[J.box];
@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(line_threads<T, CLS>(), sizeof(T) == 4 && !CLS
       if (k != 0 && 2 * k != L) row[L - k] = mk<T>(s.x + u.y, u.x - s.y);
     }
     __syncthreads();
-    const int c = threadIdx.x % W, g = threadIdx.x / W;
+    const int c = threadIdx.x & (W - 1), g = threadIdx.x >> lw;
     const bool live = c < J.nr;
     rows_pass1<T, 1, CLS>(sm + c * PX, l, g, live, tw);
     rows_pass2<T, 1, CLS>(sm + c * PX, l, g, live);

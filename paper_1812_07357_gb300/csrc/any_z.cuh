@@ -30,7 +30,7 @@ namespace psatd {
 namespace {
 
 template <typename T>
-constexpr int z_threads() {   // FP64: fewer, larger threads; its pipe needs few warps
+constexpr int z_threads() {   // at most; FP64: fewer, larger threads, its pipe needs few warps
   return sizeof(T) == 4 ? 256 : 128;
 }
 

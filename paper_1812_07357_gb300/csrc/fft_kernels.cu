@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <utility>
+#include <vector>
 
 #include "any_fft.cuh"
 #include "any_part.h"
@@ -71,18 +73,67 @@ cudaError_t configure_kernels(int prec, int smem) {
   return a != cudaSuccess ? a : b;
 }
 
-int line_tile_width(int prec) { return prec == 32 ? line_tile<float>() : line_tile<double>(); }
-
-// Shared memory, threads and class that lines of length n need, on top of
-// what c already covers (rows: x lines, else columns).
+// Shared memory, threads and class that lines of length n need in tiles of
+// 1 << c.lg, on top of what c already covers (rows: x lines, else columns).
 void line_cover(LineCfg& c, int prec, const AxisPlan& a, bool rows) {
-  const int w = line_tile_width(prec), csz = prec == 32 ? 8 : 16;
+  const int w = 1 << c.lg, csz = prec == 32 ? 8 : 16;
   const int len = !rows ? a.n : prec == 32 ? row_line_pitch(a) : (a.n + 1) | 1;
   const int r = a.r1 > a.r2 ? a.r1 : a.r2;
   c.smem = c.smem > w * len * csz ? c.smem : w * len * csz;
   const int t = (w * r + 31) / 32 * 32;
   c.threads = c.threads > t ? c.threads : t;
   if (r > 16) c.cls = 1;
+}
+
+namespace {
+// warp instructions (in lane operations) of `items` threads of `ops` operations each in blocks of nt
+double lane_ops(int items, double ops, int nt) { return (items + nt - 1) / nt * nt * ops; }
+double radix_total(int r) { return r * radix_ops(r); }
+}  // namespace
+
+// Tile of the x or y passes over `lines` (length, number of lines): FP32 16, FP64
+// the one of 8 and 16 that wastes fewer lanes in the last warp of a pass, 8
+// while 16 would leave SMs without work (`sms` x 4 tiles of six slots) and for
+// radices above 16 (registers).  90 = 9 * 10: 72 and 80 threads of 96 in tiles
+// of 8, 144 and 160 of 160 in tiles of 16.
+int line_lg(int prec, const std::vector<std::pair<AxisPlan, int64_t>>& lines, int sms) {
+  if (prec == 32) return 4;
+  double cost[2] = {0, 0};
+  int64_t total = 0;
+  for (const auto& l : lines) {
+    const AxisPlan& a = l.first;
+    if (a.r1 > 16 || a.r2 > 16) return 3;
+    for (int k = 0; k < 2; ++k) {
+      const int w = 8 << k;
+      cost[k] += (double)l.second / w *
+                 (lane_ops(w * a.r2, radix_total(a.r1), 32) + lane_ops(w * a.r1, radix_total(a.r2), 32));
+    }
+    total += l.second;
+  }
+  return total * 6 / 16 >= 4 * sms && cost[1] < 0.97 * cost[0] ? 4 : 3;
+}
+
+// Threads of a z block: FP32 256; FP64 128, or 96 where that wastes fewer lanes over
+// the passes and the update (some 190 operations per mode) of the lines of
+// `axes` and the launch fills the SMs (`tiles`; a small one needs every warp: 32^3
+// 46 us per step with 128, 48 with 64).  J form, z length 72: 128 threads run
+// 77 % full, 96 threads 95 %; with the tiles of line_lg, 8 boxes of 100 x 90 x 72
+// 6.33 -> 5.70 ms.
+void z_threads_for(LineCfg& c, int prec, int form, int nft, const std::vector<AxisPlan>& axes, int64_t tiles,
+                   int sms) {
+  c.threads = prec == 32 ? 256 : 128;
+  if (prec == 32 || tiles < 3 * sms) return;
+  const int tx = 1 << c.lg, fout = fields_out(form);
+  auto cost = [&](int nt) {
+    double v = 0;
+    for (const AxisPlan& a : axes)
+      v += (lane_ops(nft * a.r2 * tx, radix_total(a.r1), nt) + lane_ops(nft * a.r1 * tx, radix_total(a.r2), nt) +
+            lane_ops(a.n * tx, 190, nt) + lane_ops(fout * a.r1 * tx, radix_total(a.r2), nt) +
+            lane_ops(fout * a.r2 * tx, radix_total(a.r1), nt)) /
+           ((double)a.n * tx);
+    return v;
+  };
+  if (cost(96) < 0.97 * cost(128)) c.threads = 96;
 }
 
 // Columns per z tile (a power of two, its logarithm in c.lg) and the shared

@@ -265,6 +265,21 @@ std::vector<CopyBlk> build_blocks(const psatd_plan_desc* d) {
 // ---------------------------------------------------------------------------
 namespace psatd {
 
+namespace {
+const struct {
+  int r;
+  double ops;
+} kRadix[] = {{1, 0},    {2, 2},     {3, 4.67},   {4, 4},     {5, 7.2},    {6, 6.67},   {8, 7},
+              {9, 11.1}, {10, 9.2},  {12, 8.67},  {15, 11.9}, {16, 10.5},  {18, 13.1},  {20, 11.2},
+              {24, 11.7}, {25, 17},  {27, 18.5},  {30, 13.9}, {32, 13.5}};
+}  // namespace
+
+double radix_ops(int r) {
+  for (const auto& k : kRadix)
+    if (k.r == r) return k.ops;
+  return 0;
+}
+
 // Split n = r1 * r2 over the radices of the generic kernels: fewest operations
 // per point -- those of the two small DFTs (counted from the codelets: complex
 // sums, products and fused multiply-adds) and 4 per twiddle, of which coprime
@@ -273,12 +288,6 @@ namespace psatd {
 // smaller radix leaves that many lanes without work.
 // Radices above 16 cost registers and are taken where nothing else divides n.
 bool line_plan(int n, AxisPlan& ap, int prec, bool row) {
-  static const struct {
-    int r;
-    double ops;
-  } kRadix[] = {{1, 0},    {2, 2},     {3, 4.67},   {4, 4},     {5, 7.2},    {6, 6.67},   {8, 7},
-                {9, 11.1}, {10, 9.2},  {12, 8.67},  {15, 11.9}, {16, 10.5},  {18, 13.1},  {20, 11.2},
-                {24, 11.7}, {25, 17},  {27, 18.5},  {30, 13.9}, {32, 13.5}};
   auto gcd = [](int a, int b) {
     while (b) {
       const int t = a % b;
@@ -853,6 +862,19 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
       zgen.push_back(bi);
     }
   };
+  {
+    std::vector<std::pair<AxisPlan, int64_t>> lx, ly, lz;
+    for (const BoxDev& b : P->hboxes) {
+      const ShapeDev& sh = P->hshapes[b.shape];
+      lx.push_back({sh.ax, (int64_t)b.n[1] * b.n[2]});
+      ly.push_back({sh.ay, (int64_t)sh.hx * b.n[2]});
+      lz.push_back({sh.az, (int64_t)sh.hx * b.n[1]});
+    }
+    P->cfg_x.lg = line_lg(P->prec, lx, P->sms);
+    P->cfg_y.lg = line_lg(P->prec, ly, P->sms);
+    P->cfg_zonly.lg = line_lg(P->prec, lz, P->sms);
+  }
+  const int wx = 1 << P->cfg_x.lg, wy = 1 << P->cfg_y.lg, wz = 1 << P->cfg_zonly.lg;
   std::vector<RowJob> fast_rows;
   std::vector<ColJob> fast_ycols;
   for (int bi = 0; bi < (int)P->boxes.size(); ++bi) {
@@ -865,7 +887,6 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
     const int sm_zf = z_fast_smem(P->prec, P->form, n2);
     const bool fast_ok = plane_ok(b, sh);
     const int rows = n1 * n2;
-    const int nr = line_tile_width(P->prec);
     const bool pencil_ok = !(d.flags & PSATD_GENERIC_KERNELS) && P->form != kPml && sh.px >= 0 && sh.py >= 0 &&
                            sh.pz >= 0 &&
                            n2 <= pencil_max_z(P->prec) && sm_zf <= optin;
@@ -906,7 +927,7 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
       z_boxes(bi, pencil);
       for (int z = b.ng_lo[2]; z < n2 - b.ng_hi[2]; ++z) {
         const int y0 = b.ng_lo[1], y1 = n1 - b.ng_hi[1];
-        for (int y = y0; y < y1; y += nr) P->g_rows_int.push_back({bi, z * n1 + y, std::min(nr, y1 - y), 0});
+        for (int y = y0; y < y1; y += wx) P->g_rows_int.push_back({bi, z * n1 + y, std::min(wx, y1 - y), 0});
       }
     }
     line_cover(P->cfg_x, P->prec, sh.ax, true);
@@ -914,10 +935,10 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
     line_cover(P->cfg_zonly, P->prec, sh.az, false);
     // column tiles run on through the planes
     std::vector<RowJob>& rl = fast ? fast_rows : P->rows_all;
-    for (int r = 0; r < rows; r += nr) rl.push_back({bi, r, std::min(nr, rows - r), 0});
-    column_tiles(fast ? fast_ycols : P->ycols_all, bi, 0, n2, hx, nr);
-    column_tiles(P->zcols, bi, 0, n1, hx, nr);
-    if (!fast) column_tiles(P->g_ycols_int, bi, b.ng_lo[2], n2 - b.ng_hi[2], hx, nr);
+    for (int r = 0; r < rows; r += wx) rl.push_back({bi, r, std::min(wx, rows - r), 0});
+    column_tiles(fast ? fast_ycols : P->ycols_all, bi, 0, n2, hx, wy);
+    column_tiles(P->zcols, bi, 0, n1, hx, wz);
+    if (!fast) column_tiles(P->g_ycols_int, bi, b.ng_lo[2], n2 - b.ng_hi[2], hx, wy);
   }
   P->g_nrows = (int64_t)P->rows_all.size();
   P->g_nycols = (int64_t)P->ycols_all.size();
@@ -936,6 +957,15 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
     for (const psatd_box& b : P->boxes) zlongest = std::max(zlongest, b.n[2]);
   }
   z_cover(P->cfg_z, P->prec, P->form, zlongest, zcolumns, P->z_tile, P->sms, optin);
+  {
+    std::vector<AxisPlan> axes;
+    for (int bi : zgen) axes.push_back(P->hshapes[P->hboxes[bi].shape].az);
+    for (int bi = 0; zgen.empty() && bi < (int)P->boxes.size(); ++bi)
+      axes.push_back(P->hshapes[P->hboxes[bi].shape].az);
+    z_threads_for(P->cfg_z, P->prec, P->form,
+                  (d.flags & PSATD_J_CONSTANT) && P->form != kVacuum && P->form != kPml ? FIN - 3 : FIN, axes,
+                  zcolumns >> P->cfg_z.lg, P->sms);
+  }
   for (const ShapeDev& sh : P->hshapes)
     if (std::max(sh.az.r1, sh.az.r2) > 16) P->cfg_z.cls = 1;
   for (int bi : zgen)
@@ -2284,10 +2314,10 @@ psatd_status psatd_plan_distribute(psatd_plan* P, int32_t world, int32_t rank) {
     hb.push_back(rows);
     // the tile sizes of the plan's generic kernels (the same lengths, so its launches cover them)
     std::vector<RowJob> rj;
-    const int nr = line_tile_width(P->prec);
-    for (int r = 0; r < nz * n1; r += nr) rj.push_back({ib, r, std::min(nr, nz * n1 - r), 0});
+    const int wx = 1 << P->cfg_x.lg;
+    for (int r = 0; r < nz * n1; r += wx) rj.push_back({ib, r, std::min(wx, nz * n1 - r), 0});
     std::vector<ColJob> yc, zc;
-    column_tiles(yc, ib, 0, nz, hx, nr);
+    column_tiles(yc, ib, 0, nz, hx, 1 << P->cfg_y.lg);
     column_tiles(zc, ib + 1, 0, ny, hx, 1 << P->cfg_z.lg);
     CK(P, upload(P, hb, &d.d_boxes));
     CK(P, upload(P, rj, &d.d_rows));

@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cstdint>
+#include <utility>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -40,7 +41,7 @@ struct AxisPlan {
 
 // Launch of a generic kernel over lines of several lengths: the largest shared
 // memory and block any of them needs, the class of the largest radix, and the
-// logarithm of the z pass's tile width.
+// logarithm of the tile's lines.
 struct LineCfg {
   int smem = 0, threads = 0, cls = 0, lg = 0;
 };
@@ -202,14 +203,14 @@ inline void set_constants(DevPlan& P, double c, double eps0, double dt) {
 // ---- generic kernels (fft_kernels.cu, any_lines.cuh, any_z.cuh) ---------------------------
 
 // Forward R2C along x of `nf` field slots into spectrum slots (stride
-// sstride); row jobs of at most line_tile_width rows.
+// sstride); row jobs of at most 1 << c.lg rows.
 // ggrid (deferred exchange): the gather grid of every plane, box b's plane z
 // at boxes[b].gplane + z, used for the slots f < ngather; null: plain rows
 cudaError_t launch_fwd_x(int prec, const DevPlan& P, const FieldPtrs& f, int nf, void* spec, int64_t sstride,
                          const RowJob* jobs, int64_t njobs, const LineCfg& c, const GatherGrid* ggrid, int ngather,
                          cudaStream_t st);
 // Complex FFT along y (axis 1) or z (axis 2), in place on spectrum slots;
-// column jobs of at most line_tile_width columns.
+// column jobs of at most 1 << c.lg columns.
 cudaError_t launch_col(int prec, int dir, int axis, const DevPlan& P, void* spec, int64_t sstride, int nf,
                        const ColJob* jobs, int64_t njobs, const LineCfg& c, cudaStream_t st);
 // z forward FFT + k-space update + z inverse FFT, all slots of `form`; jobs of
@@ -220,7 +221,9 @@ cudaError_t launch_z_update(int prec, int form, const DevPlan& P, void* spec, in
 // C2R inverse along x with 1/(n0 n1 n2) into field slots; interior_only skips guards.
 cudaError_t launch_inv_x(int prec, const DevPlan& P, const FieldPtrs& f, int nf, void* spec, int64_t sstride,
                          const RowJob* jobs, int64_t njobs, const LineCfg& c, int interior_only, cudaStream_t st);
-int line_tile_width(int prec);   // rows or columns of a tile
+int line_lg(int prec, const std::vector<std::pair<AxisPlan, int64_t>>& lines, int sms);
+void z_threads_for(LineCfg& c, int prec, int form, int nft, const std::vector<AxisPlan>& axes, int64_t tiles,
+                   int sms);
 void line_cover(LineCfg& c, int prec, const AxisPlan& a, bool rows);
 void z_cover(LineCfg& c, int prec, int form, int n2_max, int64_t columns, int widest, int sms, int optin);
 
@@ -334,6 +337,8 @@ cudaError_t launch_z_reg_multi(int form, const DevPlan& P, void* spec, int64_t s
 int z_reg_multi_smem(int form);
 
 // ---- host helpers (plan.cpp) ------------------------------------------------
+// Operations per point of a radix of the generic kernels (0: none such).
+double radix_ops(int r);
 // Two radices and the index maps of a complex FFT length (false when there are
 // none: not 5-smooth, or above 1024).  row: an x line; FP32 rows take no
 // prime-factor maps (their lanes run along the row, which such maps scatter).

@@ -139,14 +139,16 @@ extern "C" psatd_status psatd_push_box_static(const int32_t n[3], int32_t order_
   const int64_t spec = (int64_t)hx * n1 * n2;
   std::vector<RowJob> rows;
   std::vector<ColJob> ycols, zcols;
-  const int nr = line_tile_width(32);
+  LineCfg cfx, cy, cz;
+  cfx.lg = cy.lg = line_lg(32, {}, 0);
+  const int nr = 1 << cfx.lg;
   for (int r = 0; r < n1 * n2; r += nr) rows.push_back({0, r, std::min(nr, n1 * n2 - r), 0});
   column_tiles(ycols, 0, 0, n2, hx, nr);
-  LineCfg cfx, cy, cz;
   line_cover(cfx, 32, s.ax, true);
   line_cover(cy, 32, s.ay, false);
   // a tile per SM of the largest part, so that the lists do not depend on the device
   z_cover(cz, 32, kVacuum, n2, (int64_t)n1 * hx, 0, 160, 200 * 1024);
+  z_threads_for(cz, 32, kVacuum, FIN, {s.az}, 0, 0);
   cz.cls = std::max(s.az.r1, s.az.r2) > 16;
   column_tiles(zcols, 0, 0, n1, hx, 1 << cz.lg);
   const int smem = std::max({cfx.smem, cy.smem, cz.smem});
