@@ -78,8 +78,10 @@ typedef enum {
 #define PSATD_GENERIC_KERNELS 0x10u /* diagnostics: run every box through the generic */
                                   /* kernels even where a fast path exists (the two  */
                                   /* agree to rounding)                              */
-#define PSATD_PENCIL_KERNELS 0x20u /* run every box the pencil kernels accept on     */
-                                  /* them (one kernel per axis pass)                 */
+#define PSATD_PENCIL_KERNELS 0x20u /* run every box of the pencil family on it: the  */
+                                  /* generic kernels, one per axis pass, with the    */
+                                  /* deferred exchange and, in FP32, the register z  */
+                                  /* kernels                                         */
 #define PSATD_NODAL          0x80u /* collocated variant (not in the paper, which   */
                                   /* uses staggered stencils): every component at   */
                                   /* the cell nodes, order-p centred symbol         */
@@ -91,11 +93,11 @@ typedef enum {
                                   /* the shape has register codelets).  Without      */
                                   /* either flag: plane kernels when their register- */
                                   /* resident form serves every plane-eligible box,  */
-                                  /* else pencil kernels; all families agree to      */
+                                  /* else the pencil family; all families agree to   */
                                   /* rounding                                        */
 #define PSATD_EAGER_EXCHANGE 0x100u /* store the guard cells in every step.  Without */
                                   /* it, plans whose boxes all run on the register  */
-                                  /* plane kernels (or all on the pencil kernels,   */
+                                  /* plane kernels (or all in the pencil family,    */
                                   /* when each plane's guard faces form at most 3x3 */
                                   /* rectangles) defer each step's guard exchange   */
                                   /* into the next step's forward pass, which reads */
@@ -429,10 +431,10 @@ int64_t psatd_last_launch_count(const psatd_plan* plan);
  * -1 for a NULL plan. */
 int32_t psatd_plan_fast_boxes(const psatd_plan* plan);
 
-/* Number of boxes that run on the pencil kernels (two-pass lengths up to 512
- * along x and y, up to 256 along z in FP32 / 128 in FP64, planes too large
- * for the plane kernels); the remaining boxes run on the generic multi-pass
- * kernels.  -1 for a NULL plan.  No counterpart in the paper (a property of
+/* Number of boxes of the pencil family (lengths with a fixed two-pass split, up
+ * to 512 along x and y, up to 256 along z in FP32 / 128 in FP64, planes not on
+ * the plane kernels); the remaining boxes run on the generic kernels without
+ * that family's deferred exchange and register z kernels.  -1 for a NULL plan.  No counterpart in the paper (a property of
  * this implementation's kernel selection). */
 int32_t psatd_plan_pencil_boxes(const psatd_plan* plan);
 
@@ -452,12 +454,13 @@ int32_t psatd_plan_deferred_exchange(const psatd_plan* plan);
  *                            the input tile of the CTA launched `value` blocks
  *                            after it (0 = off; 0 <= value <= 2^20;
  *                            default 64).
- *   PSATD_TUNE_PENCIL_ROWS_KB  pencil x-pass batching: shared memory (KiB)
- *                            for the rows one CTA transforms (8 .. 200;
- *                            default 64).
- *   PSATD_TUNE_Z_TILE        mx columns per tile of the shared-memory plane
- *                            family's and the pencil family's z pass (1 ..
- *                            8 in FP32, 1 .. 4 in FP64; default the maximum).
+ *   PSATD_TUNE_PENCIL_ROWS_KB  accepted (8 .. 200) and used by no kernel: rows
+ *                            go 8 or 16 to a CTA.
+ *   PSATD_TUNE_Z_TILE        most mx columns per tile of the shared-memory
+ *                            plane family's and the generic z pass (1 .. 8 in
+ *                            FP32, 1 .. 4 in FP64; the generic pass takes the
+ *                            power of two below, at least 2 in FP32; default:
+ *                            what the kernel chooses).
  *   PSATD_TUNE_HOST_COPY     (runtime) psatd_push_host's copies: 1 (default)
  *                            = a copy kernel on the SMs reading and writing
  *                            the host buffers through their device mapping
@@ -465,11 +468,12 @@ int32_t psatd_plan_deferred_exchange(const psatd_plan* plan);
  *                            16-byte aligned (else the copy engines); 0 = the
  *                            copy engines, one stream per component.
  *   PSATD_TUNE_PENCIL_REG_Z  FP32 boxes whose z length has a register z
- *                            kernel (48, 60, 80, 96, 120), on the pencil
- *                            kernels, or on the plane kernels in a batch of
- *                            several z lengths: 1 (default) = that kernel
- *                            does their z pass, 0 = the shared-memory z
- *                            kernel of their family.
+ *                            kernel (48, 60, 80, 96, 120; 128 and 192 in the
+ *                            vacuum form), in the pencil family, or on the
+ *                            plane kernels in a batch of several z lengths:
+ *                            1 (default) = that kernel does their z pass, 0 =
+ *                            the shared-memory plane z kernel or the generic
+ *                            z pass.
  *   PSATD_TUNE_Z_ONE_LAUNCH  (runtime) those boxes' z pass: 0 (default) = one
  *                            launch per z length, 1 = one persistent launch
  *                            for every z length (2 CTAs per SM, each taking

@@ -8,17 +8,17 @@ of ranks per group depends on the machine and the problem size) and leaves
 the automation for later.  Here the per-box work of one GPU is what is
 tuned:
 
-* kernel family (``PSATD_*_KERNELS``): plane kernels, pencil kernels or
-  generic kernels, for the boxes each family takes;
+* kernel family (``PSATD_*_KERNELS``): plane kernels, the pencil family or the
+  plain generic kernels, for the boxes each family takes;
 * ``reg_planes``: the register plane kernels for the FP32 boxes whose plane
   shape has them, or the family those boxes take without them;
-* ``z_tile``: mx columns per z tile of the plane and pencil families (more,
+* ``z_tile``: most mx columns per z tile of the plane and pencil families (more,
   smaller CTAs for small boxes);
-* ``pencil_rows_kb``: pencil batching -- the shared memory, hence the number
-  of x rows, of one pencil CTA;
+* ``pencil_rows_kb``: searched only while a plan reports it; no kernel of this
+  version does;
 * ``z_prefetch``: the register z kernel's L2 prefetch distance;
-* ``pencil_reg_z``: the register z kernel or the shared-memory one for the z
-  pass of pencil boxes whose z length has both;
+* ``pencil_reg_z``: the register z kernel or the shared-memory / generic one for
+  the z pass of pencil boxes whose z length has both;
 * ``z_one_launch``: those boxes' z pass in one persistent launch for every z
   length, or one launch per length.
 

@@ -1,4 +1,4 @@
-// Building blocks of the fast and pencil FFT kernels: two-pass ("four-step")
+// Building blocks of the shared-memory plane kernels: two-pass ("four-step")
 // transforms of columns held in shared memory, asynchronous row copies, and
 // the fused z pass (z FFT of every field slot of a tile of mx columns, the
 // k-space update, the inverse z FFT of the output slots).

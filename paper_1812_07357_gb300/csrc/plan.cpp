@@ -823,10 +823,10 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
   const int tile = P->z_tile > 0 ? std::min(P->z_tile, fast_tile(P->prec)) : fast_tile(P->prec);
   // Kernel family of each box: plane kernels (x+y per z plane) for the boxes
   // whose plane shape has register-resident plane kernels (FP32, one launch
-  // per shape); otherwise the pencil kernels (one launch per axis and FFT
-  // length) take the boxes they accept, which measured faster than the
-  // shared-memory plane kernels on mixed batches; the rest run on the
-  // generic kernels.  PSATD_PENCIL_KERNELS and PSATD_PLANE_KERNELS
+  // per shape); otherwise the pencil family (the generic kernels with the
+  // deferred exchange and, in FP32, the register z kernels) takes the boxes it
+  // accepts, which measured faster than the shared-memory plane kernels on
+  // mixed batches; the rest run on the plain generic kernels.  PSATD_PENCIL_KERNELS and PSATD_PLANE_KERNELS
   // prefer one family outright, PSATD_GENERIC_KERNELS the generic kernels.
   auto plane_ok = [&](const psatd_box& b, const ShapeDev& sh) {
     const int L = b.n[0] / 2, n1 = b.n[1], n2 = b.n[2], hx = L + 1;
@@ -970,7 +970,7 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
     if (std::max(sh.az.r1, sh.az.r2) > 16) P->cfg_z.cls = 1;
   for (int bi : zgen)
     column_tiles(P->g_zcols, bi, 0, P->boxes[bi].n[1], P->boxes[bi].n[0] / 2 + 1, 1 << P->cfg_z.lg);
-  // pencil jobs grouped by the FFT length of the axis each kernel transforms
+  // jobs grouped by what a kernel is instantiated for (plane shape, z length)
   // (one launch per group; boxes keep their order inside a group)
   auto group = [&](auto& list, auto code_of, std::vector<psatd_plan::Group>& groups) {
     std::stable_sort(list.begin(), list.end(),

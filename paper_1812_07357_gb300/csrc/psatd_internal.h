@@ -12,7 +12,7 @@
 
 namespace psatd {
 
-constexpr int kThreads = 256;      // threads per CTA of the plane and pencil z kernels
+constexpr int kThreads = 256;      // threads per CTA of the shared-memory plane z kernel
 
 // Equation form of the k-space update (slot layout of the fields):
 //   kVacuum: E 0-2, B 3-5                      (6 in, 6 out)
@@ -20,7 +20,7 @@ constexpr int kThreads = 256;      // threads per CTA of the plane and pencil z 
 //   kRhoForm: E 0-2, B 3-5, rho 6, J 7-9       (10 in, 7 out)
 //   kPml   : E 0-2, B 3-5 in; E, B and the increments of the stored split
 //            parts E_xy, E_yz, E_zx, B_xy, B_yz, B_zx in 6-11 out (vacuum
-//            with absorbing layers; generic kernels only)
+//            with absorbing layers; generic z pass only)
 enum Form { kVacuum = 0, kJForm = 1, kRhoForm = 2, kPml = 3 };
 
 constexpr int fields_in(int form) { return form == kVacuum || form == kPml ? 6 : form == kJForm ? 9 : 10; }
