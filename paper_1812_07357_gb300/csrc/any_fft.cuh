@@ -48,12 +48,12 @@ __device__ __forceinline__ int line_lg(int lg) {
 // bank conflicts; the natural-order row needs r1 * r2 of it.
 __host__ __device__ __forceinline__ int row_line_pitch(const AxisPlan& a) { return a.r1 * (a.r2 | 1); }
 
-// complex elements between two slots of a z tile: n2 * tx and a pad that makes
-// the pitch half a 128-byte line (mod 128 bytes)
+// complex elements between two slots of a z tile: n2 * tx and a pad that puts
+// each slot one row (tx columns) further within a 128-byte line, so that lanes
+// over (column, slot) read different banks whatever the tile's width
 __host__ __device__ constexpr int z_slot_pitch(int csz, int n2, int tx) {
-  const int half = 64 / csz, line = 128 / csz;
-  const int p = n2 * tx;
-  return p + (half + line - p % line) % line;
+  const int line = 128 / csz, p = n2 * tx;
+  return p + (tx % line + line - p % line) % line;
 }
 
 // Threads of a block at most: a tile times the largest radix of the class

@@ -10,9 +10,9 @@
 // p = (k1, k2) of a line holds frequency (a_out k1 + s_out k2) mod n2), then
 // the same two passes mirrored, the last one straight back to HBM.  So no pass
 // permutes its line and a block waits at four barriers.  Shared memory is
-// [slot][place][column], the slots half a 128-byte line apart, so that lanes
-// over (column, place) and lanes over (column, slot) both read it without
-// bank conflicts.
+// [slot][place][column], each slot a row further within a 128-byte line than the
+// one before, so that lanes over (column, place) and lanes over (column, slot)
+// both read it without bank conflicts.
 #pragma once
 
 #include <cuda_runtime.h>
