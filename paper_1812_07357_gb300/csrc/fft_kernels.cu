@@ -67,10 +67,12 @@ cudaError_t launch_z_update(int prec, int form, const DevPlan& P, void* spec, in
                   [&](auto p, dim3 g) { p.z_update(g, form, P, spec, sstride, jobs, c, nft, st); });
 }
 
-cudaError_t configure_kernels(int prec, int smem) {
-  const cudaError_t a = prec == 32 ? AnyPart<float, 0>::configure(smem) : AnyPart<double, 0>::configure(smem);
-  const cudaError_t b = prec == 32 ? AnyPart<float, 1>::configure(smem) : AnyPart<double, 1>::configure(smem);
-  return a != cudaSuccess ? a : b;
+cudaError_t configure_kernels(int prec, int smem, int classes) {
+  cudaError_t e = cudaSuccess;
+  if (classes & 1) e = prec == 32 ? AnyPart<float, 0>::configure(smem) : AnyPart<double, 0>::configure(smem);
+  if (e == cudaSuccess && (classes & 2))
+    e = prec == 32 ? AnyPart<float, 1>::configure(smem) : AnyPart<double, 1>::configure(smem);
+  return e;
 }
 
 // Shared memory, threads and class that lines of length n need in tiles of

@@ -1220,7 +1220,9 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
   if (smem > optin) return fail(P, PSATD_ERR_UNSUPPORTED_SIZE, fmt("needs %d B shared memory", smem));
   // The attribute is a per-kernel cap shared by every plan: raise it to the
   // device maximum so that no plan lowers it below another plan's need.
-  CK(P, configure_kernels(P->prec, optin));
+  int classes = 0;
+  for (const LineCfg* c : {&P->cfg_x, &P->cfg_y, &P->cfg_zonly, &P->cfg_z}) classes |= 1 << c->cls;
+  CK(P, configure_kernels(P->prec, optin, classes));
   CK(P, configure_fast_kernels(P->prec, optin));
   if (P->prec == 32) CK(P, configure_reg_kernels(optin));
   if (P->fast_boxes) {

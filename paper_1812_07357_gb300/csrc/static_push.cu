@@ -205,7 +205,7 @@ extern "C" psatd_status psatd_push_box_static(const int32_t n[3], int32_t order_
       return err(PSATD_ERR_UNSUPPORTED_SIZE, "box needs %d B of shared memory per block; the device allows %d B",
                  smem, optin);
     if (!g_configured[dev]) {
-      e = configure_kernels(32, optin);
+      e = configure_kernels(32, optin, 3);
       if (e != cudaSuccess) return err(PSATD_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
       g_configured[dev] = true;
     }
