@@ -7,10 +7,20 @@
 //              (grid_order).  For a launch whose predecessor is a single
 //              launch of the same call, so that its end is the end of all work
 //              before it.
-//   kBeside    starts while the launch before it drains and does not wait: for
-//              the second and later launches of one pass over different
-//              boxes, the first of which is kOrdinary.  The launch after the
-//              pass is kOrdinary again.
+//   kBeside    starts while the launch before it drains and computes beside it:
+//              for the second and later launches of one pass over different
+//              boxes, the first of which is kOrdinary.  Its grid has one block (or
+//              cluster) more than it has work, which only waits for that launch
+//              to finish (grid_join), so the end of each launch of the pass
+//              implies the end of the one before it.  The launch after the pass is
+//              kOrdinary again.  That wait is what orders the pass in a CUDA graph, whose
+//              only full edge into the next pass comes from the pass's last
+//              launch (a stream would wait for all of them).  It always ends: a
+//              launch starts beside another only when every block of that one
+//              has started.  A block of its own, tested for behind the loads of
+//              the job: 128 boxes of 96^3 2.864 ms per step, against 2.860
+//              without any of it, 2.870 with the test first and 2.909 with a
+//              wait of block 0 at the end of every kernel, which changed their code.
 //
 // Every kernel here lets its successor start as soon as all its own blocks have
 // (grid_release), so a successor's blocks only take the room that the last
@@ -23,7 +33,7 @@
 // their small L1 (128 boxes of 96^3: 2.90 -> 3.22 ms per step).  Not captured
 // steps: 32^3 FP64 45 -> 56 us per step.  Beside: the register kernels of a batch
 // of many box shapes, 60 launches a step whose tails overlap (40 uneven boxes
-// 1.51 -> 1.27 ms per step).
+// 1.51 -> 1.28 ms per step).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -36,6 +46,19 @@ __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.la
 __device__ __forceinline__ void grid_order(int order) {
   grid_release();
   if (order == kChained) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// Whether this block of a kBeside launch is one of the last `n`, which only
+// wait (grid_join).
+__device__ __forceinline__ bool grid_extra(int order, unsigned n = 1) {
+  return order == kBeside && blockIdx.x + n >= gridDim.x;
+}
+__device__ __forceinline__ void grid_join() {
+  grid_release();
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// The grid of a launch of `blocks` blocks per y index, and the extra ones when kBeside.
+inline dim3 ordered_grid(int order, unsigned blocks, unsigned y, unsigned n = 1) {
+  return dim3(blocks + (order == kBeside ? n : 0u), y);
 }
 
 template <typename... P, typename... A>

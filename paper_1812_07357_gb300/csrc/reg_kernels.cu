@@ -218,6 +218,7 @@ template <int NZ, int FORM, int ZST>
 __global__ void __launch_bounds__(z_reg_threads<FORM>(), z_reg_min_blocks<FORM>())
     k_z_reg(DevPlan P, float2* spec, int64_t sstride, const ColJob* __restrict__ jobs, int nft, int njobs,
             int pf_dist) {
+  if (grid_extra(P.order)) return grid_join();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const ColJob J = jobs[blockIdx.x];
   grid_release();
@@ -370,6 +371,7 @@ template <int NZ, int FORM>
 __global__ void __launch_bounds__(z_reg4_threads<FORM>(), 2)
     k_z_reg4(DevPlan P, float2* spec, int64_t sstride, const ColJob* __restrict__ jobs, int nft, int njobs,
              int pf_dist) {
+  if (grid_extra(P.order)) return grid_join();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const ColJob J = jobs[blockIdx.x];
   grid_release();
@@ -467,7 +469,7 @@ constexpr int kRegZst = 96 * 49;
 cudaError_t launch_z_reg(int form, const DevPlan& P, void* spec, int64_t sstride, const ColJob* jobs,
                          int64_t njobs, int n2, int zst, int nft, int pf_dist, cudaStream_t st) {
   if (njobs <= 0) return cudaSuccess;
-  dim3 grid((unsigned)njobs);
+  const dim3 grid = ordered_grid(P.order, (unsigned)njobs, 1);
   const int smem = z_reg_smem(form, n2);
 #define PSATD_ZF(NZV, F, ZS)                                                                      \
   launch_ordered(P.order, k_z_reg<NZV, F, ZS>, grid, z_reg_threads<F>(), smem, st, P, (float2*)spec, \

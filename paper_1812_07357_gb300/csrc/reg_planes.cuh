@@ -150,10 +150,12 @@ __global__ void __launch_bounds__(reg_plane_threads<L, NY>(), reg_plane_min_bloc
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ float2 wsc[NY];   // y transform of the packed real columns
   float* buf = reinterpret_cast<float*>(smem_raw);
-  const int2 J = jobs[blockIdx.x];
+  const bool extra = grid_extra(P.order);
+  const int2 J = jobs[blockIdx.x - extra];   // an extra block makes no use of it
   const int f = blockIdx.y;
   const BoxDev bx = P.boxes[J.x];
   grid_release();
+  if (extra) return grid_join();
   plane_load<N0, NY, NT>(P, F, buf, J, f, bx, gstart, gsegs, ggrid, ngather);
   // x: row r -> half spectrum X[0..L] written back into the same row
   if (threadIdx.x < NY) {
@@ -276,10 +278,12 @@ __global__ void __launch_bounds__(reg_plane_threads<L, NY>(), reg_plane_min_bloc
   // consumed, the interior rows (pitch PF floats): X values, then real cells
   float2* sp = reinterpret_cast<float2*>(smem_raw);
   float* rows = reinterpret_cast<float*>(smem_raw);
-  const int2 J = jobs[blockIdx.x];
+  const bool extra = grid_extra(P.order);
+  const int2 J = jobs[blockIdx.x - extra];   // an extra block makes no use of it
   const int f = blockIdx.y;
   const BoxDev bx = P.boxes[J.x];
   grid_release();
+  if (extra) return grid_join();
   const int ylo = bx.ng_lo[1], yhi = NY - bx.ng_hi[1], ni = yhi - ylo;
   const int xlo = bx.ng_lo[0], nxi = N0 - bx.ng_lo[0] - bx.ng_hi[0];
   const float2* g = spec + f * sstride + bx.soff + (int64_t)J.y * NY * HX;
@@ -422,10 +426,12 @@ __global__ void __launch_bounds__(wide_threads<L, NY>(), wide_min_blocks<L, NY>(
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* buf = reinterpret_cast<float*>(smem_raw);
   float2* cb = reinterpret_cast<float2*>(smem_raw);
-  const int2 J = jobs[blockIdx.x];
+  const bool extra = grid_extra(P.order);
+  const int2 J = jobs[blockIdx.x - extra];   // an extra block makes no use of it
   const int f = blockIdx.y;
   const BoxDev bx = P.boxes[J.x];
   grid_release();
+  if (extra) return grid_join();
   plane_load<N0, NY, NT>(P, F, buf, J, f, bx, gstart, gsegs, ggrid, ngather);
   const int t = threadIdx.x;
   // x, stage 1: thread (row r, q): DFT of the packed samples z[q + GX j]
@@ -568,10 +574,12 @@ __global__ void __launch_bounds__(wide_threads<L, NY>(), wide_min_blocks<L, NY>(
   float2* sp = reinterpret_cast<float2*>(smem_raw);
   float2* cb = reinterpret_cast<float2*>(smem_raw);
   float* rows = reinterpret_cast<float*>(smem_raw);
-  const int2 J = jobs[blockIdx.x];
+  const bool extra = grid_extra(P.order);
+  const int2 J = jobs[blockIdx.x - extra];   // an extra block makes no use of it
   const int f = blockIdx.y;
   const BoxDev bx = P.boxes[J.x];
   grid_release();
+  if (extra) return grid_join();
   const int ylo = bx.ng_lo[1], yhi = NY - bx.ng_hi[1], ni = yhi - ylo;
   const int xlo = bx.ng_lo[0], nxi = N0 - bx.ng_lo[0] - bx.ng_hi[0];
   {
@@ -810,6 +818,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split_threads<L, NY>
     k_plane_fwd_split(DevPlan P, FieldPtrs F, float2* spec, int64_t sstride, const int2* __restrict__ jobs,
                       const int* __restrict__ gstart, const GatherSeg* __restrict__ gsegs,
                       const GatherGrid* __restrict__ ggrid, int ngather) {
+  if (grid_extra(P.order, 2)) return grid_join();
   constexpr int N0 = 2 * L, HX = L + 1, PF = row_pitch(N0), PC = PF / 2;
   constexpr int GX = wide_gx<L, NY>(), GY = wide_gy<L, NY>(), NT = split_threads<L, NY>();
   constexpr int LX = L / GX, LY = NY / GY, LXP = GX > 1 ? LX + 1 : LX;
@@ -974,14 +983,14 @@ bool plane_fwd_shape(int code, dim3 grid, const DevPlan& P, const FieldPtrs& f, 
   if constexpr (PART == PSATD_PLANE_PART) {
     if (code != CODE) return false;
     if constexpr (plane_is_split<L, NY>())
-      launch_ordered(P.order, k_plane_fwd_split<L, NY>, dim3(2 * grid.x, grid.y), split_threads<L, NY>(), split_smem<L, NY>(),
-                     st, P, f, (float2*)spec, sstride, jobs, gstart, gsegs, ggrid, ngather);
+      launch_ordered(P.order, k_plane_fwd_split<L, NY>, ordered_grid(P.order, 2 * grid.x, grid.y, 2),
+                     split_threads<L, NY>(), split_smem<L, NY>(), st, P, f, (float2*)spec, sstride, jobs, gstart, gsegs, ggrid, ngather);
     else if constexpr (plane_is_wide<L, NY>())
-      launch_ordered(P.order, k_plane_fwd_wide<L, NY>, grid, wide_threads<L, NY>(), plane_fwd_bytes<L, NY>(),
-                     st, P, f, (float2*)spec, sstride, jobs, gstart, gsegs, ggrid, ngather);
+      launch_ordered(P.order, k_plane_fwd_wide<L, NY>, ordered_grid(P.order, grid.x, grid.y),
+                     wide_threads<L, NY>(), plane_fwd_bytes<L, NY>(), st, P, f, (float2*)spec, sstride, jobs, gstart, gsegs, ggrid, ngather);
     else
-      launch_ordered(P.order, k_plane_fwd_reg<L, NY>, grid, reg_plane_threads<L, NY>(), plane_fwd_bytes<L, NY>(),
-                     st, P, f, (float2*)spec, sstride, jobs, gstart, gsegs, ggrid, ngather);
+      launch_ordered(P.order, k_plane_fwd_reg<L, NY>, ordered_grid(P.order, grid.x, grid.y),
+                     reg_plane_threads<L, NY>(), plane_fwd_bytes<L, NY>(), st, P, f, (float2*)spec, sstride, jobs, gstart, gsegs, ggrid, ngather);
     return true;
   } else {
     return false;
@@ -994,11 +1003,11 @@ bool plane_inv_shape(int code, dim3 grid, const DevPlan& P, const FieldPtrs& f, 
   if constexpr (PART == PSATD_PLANE_PART) {
     if (code != CODE) return false;
     if constexpr (plane_is_wide<L, NY>())
-      launch_ordered(P.order, k_plane_inv_wide<L, NY>, grid, wide_threads<L, NY>(), plane_inv_bytes<L, NY>(),
-                     st, P, f, (const float2*)spec, sstride, jobs, seg_start, segs);
+      launch_ordered(P.order, k_plane_inv_wide<L, NY>, ordered_grid(P.order, grid.x, grid.y),
+                     wide_threads<L, NY>(), plane_inv_bytes<L, NY>(), st, P, f, (const float2*)spec, sstride, jobs, seg_start, segs);
     else
-      launch_ordered(P.order, k_plane_inv_reg<L, NY>, grid, reg_plane_threads<L, NY>(), plane_inv_bytes<L, NY>(),
-                     st, P, f, (const float2*)spec, sstride, jobs, seg_start, segs);
+      launch_ordered(P.order, k_plane_inv_reg<L, NY>, ordered_grid(P.order, grid.x, grid.y),
+                     reg_plane_threads<L, NY>(), plane_inv_bytes<L, NY>(), st, P, f, (const float2*)spec, sstride, jobs, seg_start, segs);
     return true;
   } else {
     return false;
