@@ -726,9 +726,16 @@ static void build_gather(psatd_plan* P, const std::vector<char>& box_fast, uint3
   P->deferred = true;
 }
 
+// Field slots each step transforms: with PSATD_J_CONSTANT the current's
+// three slots (the last ones) keep the spectrum computed once per push.  The
+// forms without a current, absorbing layers among them, transform every slot.
+static int step_slots(const psatd_plan* P) {
+  const int FIN = fields_in(P->form);
+  return (P->desc.flags & PSATD_J_CONSTANT) && (P->form == kJForm || P->form == kRhoForm) ? FIN - 3 : FIN;
+}
+
 psatd_status build(psatd_plan* P, cudaStream_t st) {
   const psatd_plan_desc& d = P->desc;
-  const int FIN = fields_in(P->form);
   // ---- shapes and table pool layout
   std::map<std::tuple<int, int, int, int>, int> shape_of;
   std::map<int, int64_t> tw_of;  // length -> complex pool offset
@@ -962,9 +969,7 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
     for (int bi : zgen) axes.push_back(P->hshapes[P->hboxes[bi].shape].az);
     for (int bi = 0; zgen.empty() && bi < (int)P->boxes.size(); ++bi)
       axes.push_back(P->hshapes[P->hboxes[bi].shape].az);
-    z_threads_for(P->cfg_z, P->prec, P->form,
-                  (d.flags & PSATD_J_CONSTANT) && P->form != kVacuum && P->form != kPml ? FIN - 3 : FIN, axes,
-                  zcolumns >> P->cfg_z.lg, P->sms);
+    z_threads_for(P->cfg_z, P->prec, P->form, step_slots(P), axes, zcolumns >> P->cfg_z.lg, P->sms);
   }
   for (const ShapeDev& sh : P->hshapes)
     if (std::max(sh.az.r1, sh.az.r2) > 16) P->cfg_z.cls = 1;
@@ -1738,13 +1743,6 @@ static psatd_status forward_xy(psatd_plan* P, const DevPlan& D0, const FieldPtrs
   }
   *launches_out += launches;
   return PSATD_OK;
-}
-
-// Field slots each step transforms: with PSATD_J_CONSTANT the current's
-// three slots (the last ones) keep the spectrum computed once per push.
-static int step_slots(const psatd_plan* P) {
-  const int FIN = fields_in(P->form);
-  return (P->desc.flags & PSATD_J_CONSTANT) && P->form != kVacuum ? FIN - 3 : FIN;
 }
 
 // The whole 3D spectrum of the (constant) current into its workspace slots.
