@@ -154,7 +154,11 @@ extern "C" psatd_status psatd_push_box_static(const int32_t n[3], int32_t order_
   const int smem = std::max({cfx.smem, cy.smem, cz.smem});
   const std::vector<double> alpha = order_p ? stencil_alpha(order_p) : std::vector<double>(1, 0.0);
 
-  // ---- carve the arena: [box][shape][rows][ycols][zcols][alpha][r32][c32][q32][r64][c64][q64][spectra]
+  // ---- carve the arena: [box][shape][rows][ycols][zcols][alpha][r32][c32][q32][r64][q64][spectra].
+  // The FP64 twiddles and phases lie at the head of the spectra, which no kernel
+  // writes before they are rounded: the lists of 16 rows and columns a job are
+  // longer than those the limit was set for, and the boxes up to it (162 x 270 x
+  // 50) still have to fit.
   size_t off = 0;
   auto carve = [&](size_t bytes) {
     off = up(off, 256);
@@ -168,8 +172,8 @@ extern "C" psatd_status psatd_push_box_static(const int32_t n[3], int32_t order_
   const size_t o_zcols = carve(zcols.size() * sizeof(ColJob));
   const size_t o_alpha = carve(alpha.size() * sizeof(double));
   const size_t o_r32 = carve(rtot * 4), o_c32 = carve(ctot * 8), o_q32 = carve(qtot * 16);
-  const size_t o_r64 = carve(rtot * 8), o_c64 = carve(ctot * 16), o_q64 = carve(qtot * 32);
-  const size_t o_ws = carve((size_t)FIN * spec * 8);
+  const size_t o_r64 = carve(rtot * 8), o_q64 = carve(qtot * 32);
+  const size_t o_ws = carve((size_t)FIN * spec * 8), o_c64 = o_ws;
   if (off > kStaticScratchBytes)
     return err(PSATD_ERR_UNSUPPORTED_SIZE,
                "box %dx%dx%d needs %zu bytes of static scratch; the limit is %zu bytes", n0, n1, n2, off,
