@@ -454,8 +454,9 @@ int32_t psatd_plan_deferred_exchange(const psatd_plan* plan);
  *                            the input tile of the CTA launched `value` blocks
  *                            after it (0 = off; 0 <= value <= 2^20;
  *                            default 64).
- *   PSATD_TUNE_PENCIL_ROWS_KB  accepted (8 .. 200) and used by no kernel: rows
- *                            go 8 or 16 to a CTA.
+ *   PSATD_TUNE_PENCIL_ROWS_KB  kept and reported for plans with boxes of the
+ *                            pencil family (8 .. 200; default 64), used by no
+ *                            kernel: rows go 8 or 16 to a CTA.
  *   PSATD_TUNE_Z_TILE        most mx columns per tile of the shared-memory
  *                            plane family's and the generic z pass (1 .. 8 in
  *                            FP32, 1 .. 4 in FP64; the generic pass takes the

@@ -14,8 +14,8 @@ tuned:
   shape has them, or the family those boxes take without them;
 * ``z_tile``: most mx columns per z tile of the plane and pencil families (more,
   smaller CTAs for small boxes);
-* ``pencil_rows_kb``: searched only while a plan reports it; no kernel of this
-  version does;
+* ``pencil_rows_kb``: searched when a measurement reports it.  Plans keep it, but
+  no kernel uses it, so ``gpu_measure`` leaves it out;
 * ``z_prefetch``: the register z kernel's L2 prefetch distance;
 * ``pencil_reg_z``: the register z kernel or the shared-memory / generic one for
   the z pass of pencil boxes whose z length has both;
@@ -47,6 +47,7 @@ KNOB_VALUES = {
     "pencil_rows_kb": (16, 32, 64, 128),
     "z_prefetch": (0, 64, 152),
 }
+UNUSED_KNOBS = ("pencil_rows_kb",)   # reported by plans, used by no kernel
 
 
 def default_cache() -> str:
@@ -144,7 +145,7 @@ def gpu_measure(layout, h, dt, *, precision=32, sources="vacuum", nodal=False, s
                 plan.push(f, s, steps)
                 e1.record(plan.stream)
             torch.cuda.synchronize()
-            return e0.elapsed_time(e1) / steps, plan.tuning()
+            return e0.elapsed_time(e1) / steps, {k: v for k, v in plan.tuning().items() if k not in UNUSED_KNOBS}
         finally:
             plan.close()
 

@@ -428,6 +428,7 @@ struct psatd_plan {
   int reg_zst = 0;                             // n1 * (n0/2 + 1) of every register-z box, else 0
   int z_prefetch = 64;                         // register z kernel: L2 prefetch distance in CTAs (64: measured
                                                // best of 0 .. 1216 on 512 boxes of 96^3)
+  int pen_rows_kb = 64;                        // kept for psatd_plan_tuning; no kernel uses it
   int host_copy = 1;                           // host path: 1 = SM copy kernel on mapped memory, 0 = copy engines
   int z_tile = 0;                              // plane/pencil z tile columns (0: the kernel maximum)
   // absorbing layers (form kPml): the description, boxes with layer cells,
@@ -1569,6 +1570,7 @@ psatd_status psatd_plan_create(const psatd_plan_desc* desc, void* stream, psatd_
     for (int i = 0; desc->tuning && i < 16 && desc->tuning[2 * i] != 0; ++i) {
       const int32_t k = desc->tuning[2 * i], v = desc->tuning[2 * i + 1];
       if (k == PSATD_TUNE_Z_PREFETCH) P->z_prefetch = v;
+      if (k == PSATD_TUNE_PENCIL_ROWS_KB) P->pen_rows_kb = v;
       if (k == PSATD_TUNE_Z_TILE) P->z_tile = v;
       if (k == PSATD_TUNE_HOST_COPY) P->host_copy = v;
       if (k == PSATD_TUNE_PENCIL_REG_Z) P->pen_reg_z = v;
@@ -2480,7 +2482,7 @@ int32_t psatd_plan_tuning(const psatd_plan* P, int32_t knob) {
     case PSATD_TUNE_Z_PREFETCH:
       return P->reg_z || !P->zpen_reg.empty() ? P->z_prefetch : -1;
     case PSATD_TUNE_PENCIL_ROWS_KB:
-      return -1;   // accepted, used by no kernel
+      return P->pen_boxes ? P->pen_rows_kb : -1;
     case PSATD_TUNE_HOST_COPY:
       return P->host_copy;
     case PSATD_TUNE_PENCIL_REG_Z:
