@@ -82,14 +82,18 @@ __device__ __forceinline__ void rows_pass2(cx<T>* row, const Line& l, int k1, bo
   __syncthreads();
 }
 
-// Pass 1 along rows, in place.
+// Pass 1 along rows, in place: sub-transforms n2, n2 + gs, ... (class 0: a thread
+// for each).
 template <typename T, int DIR, int CLS>
-__device__ __forceinline__ void rows_pass1(cx<T>* row, const Line& l, int n2, bool live,
+__device__ __forceinline__ void rows_pass1(cx<T>* row, const Line& l, int n2, int gs, bool live,
                                            const cx<T>* __restrict__ tw) {
   if (live && n2 < l.r2)
     with_radix<CLS>(l.r1, [&](auto rc) {
-      line_pass1<T, decltype(rc)::value, DIR, true>(
-          l, n2, tw, [&](int i) { return row[i]; }, [&](int, int i, cx<T> v) { row[i] = v; });
+      do {
+        line_pass1<T, decltype(rc)::value, DIR, true>(
+            l, n2, tw, [&](int i) { return row[i]; }, [&](int, int i, cx<T> v) { row[i] = v; });
+        n2 += gs;
+      } while (CLS && n2 < l.r2);
     });
   __syncthreads();
 }
@@ -215,7 +219,7 @@ __global__ void __launch_bounds__(line_threads<T, CLS>())
     __syncthreads();
     const int c = threadIdx.x & (W - 1), g = threadIdx.x >> lw;
     const bool live = c < J.nr;
-    rows_pass1<T, -1, CLS>(sm + c * PX, l, g, live, tw);
+    rows_pass1<T, -1, CLS>(sm + c * PX, l, g, blockDim.x >> lw, live, tw);
     rows_pass2<T, -1, CLS>(sm + c * PX, l, g, live);
     split_rows<T>(sm, PX, J.nr, L, cpool<T>(P) + sh.post, out);
   }
@@ -368,7 +372,7 @@ __global__ void __launch_bounds__(line_threads<T, CLS>(), sizeof(T) == 4 && !CLS
     __syncthreads();
     const int c = threadIdx.x & (W - 1), g = threadIdx.x >> lw;
     const bool live = c < J.nr;
-    rows_pass1<T, 1, CLS>(sm + c * PX, l, g, live, tw);
+    rows_pass1<T, 1, CLS>(sm + c * PX, l, g, blockDim.x >> lw, live, tw);
     rows_pass2<T, 1, CLS>(sm + c * PX, l, g, live);
     if (pairs) {
       const int np = nxi / 2;

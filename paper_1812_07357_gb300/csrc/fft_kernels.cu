@@ -85,7 +85,14 @@ void line_cover(LineCfg& c, int prec, const AxisPlan& a, bool rows) {
   // columns of radices above 16 (112 registers): two sub-transforms per thread, so
   // that two or three blocks fit an SM (forward + inverse FFT of 240 x 200 x 180,
   // 200 = 10 * 20: 173 -> 153 us)
-  const int items = !rows && r > 16 ? (r + 1) / 2 : r;
+  int items = !rows && r > 16 ? (r + 1) / 2 : r;
+  // FP64 rows of radices above 16 (252 registers): 128 threads where they hold pass
+  // 2, a thread per sub-transform of the smaller radix (line_plan puts it first),
+  // so that two blocks fit an SM and one computes while the other loads; pass 1
+  // loops.  250^3 vacuum 27.6 -> 23.2 ms per step, 324 x 96 x 96 rho form 4.75 ->
+  // 4.23, 500 x 96 x 96 7.25 -> 6.69.  Above 128 one block fits either way and
+  // needs its warps: 1000 x 64 x 64 6.01 ms with 224 threads, 6.44 with 160.
+  if (rows && prec == 64 && r > 16 && w * a.r1 <= 128) items = 128 / w;
   const int t = (w * items + 31) / 32 * 32;
   c.threads = c.threads > t ? c.threads : t;
   if (r > 16) c.cls = 1;
