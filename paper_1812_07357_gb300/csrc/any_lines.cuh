@@ -30,12 +30,12 @@
 // What bounds them: FP64 the two FP64 lanes of an SM (84 % busy), FP32 memory
 // latency and instruction issue.  Measured on GB300 against radix-8 Stockham
 // passes in shared memory (two barriers per pass, run-time modulo per butterfly,
-// 4096 points per block): absorbing layers, 8 boxes of 96^3 FP32 4.19 -> 0.68 ms
-// per step; FP64 J form, 8 boxes of 100 x 90 x 72 8.53 -> 6.35 ms; forward +
-// inverse FFT of 240 x 200 x 180 FP32 858 -> 183 us; 32^3 FP64 157 -> 46 us per
-// step.  Against a kernel per length with whole tiles staged in shared memory:
-// two FP32 boxes of 384 x 256 x 256 3.74 -> 3.27 ms per step, 160 x 120 x 128
-// FP32 213 -> 170 us, 128^3 FP64 rho form 3.03 -> 2.63 ms.
+// 4096 points per block): a 100 x 90 x 80 box with absorbing layers FP32 726 ->
+// 119 us per step; FP64 J form, 8 boxes of 100 x 90 x 72 8.52 -> 5.70 ms; forward +
+// inverse FFT of 240 x 200 x 180 FP32 with a filter between 856 -> 152 us; 32^3 FP64
+// 157 -> 46 us per step.  Against a kernel per length with whole tiles staged in
+// shared memory: two FP32 boxes of 384 x 256 x 256 3.74 -> 2.92 ms per step, 256^3
+// FP32 1.33 -> 1.05, 128^3 FP64 rho form 3.03 -> 2.61.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -895,6 +895,8 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
     const int sm_zf = z_fast_smem(P->prec, P->form, n2);
     const bool fast_ok = plane_ok(b, sh);
     const int rows = n1 * n2;
+    // (lengths and limits of kernels the family had before the generic ones; they
+    // still say which boxes defer the exchange and take a register z kernel)
     const bool pencil_ok = !(d.flags & PSATD_GENERIC_KERNELS) && P->form != kPml && sh.px >= 0 && sh.py >= 0 &&
                            sh.pz >= 0 &&
                            n2 <= pencil_max_z(P->prec) && sm_zf <= optin;

@@ -270,9 +270,10 @@ __global__ void __launch_bounds__(z_reg_threads<FORM>(), z_reg_min_blocks<FORM>(
 // the half-length spectrum of their half (rows of the pair kernel's layout),
 // the update stage is the pair kernel's, and the inverse mirrors the forward
 // (split by shuffles, length-NZ/4 inverse DFTs, interior z planes stored).
-// The vacuum form only: with 9 or 10 slots its tiles have 4 columns, and the
-// generic z pass (8 columns) is faster (8 boxes of 192^3: J form 4.48 -> 4.04 ms
-// per step, rho form 4.99 -> 4.71; vacuum 2.93 against 3.00).
+// Instantiated for the vacuum form only: with 9 or 10 slots it ran tiles of 4
+// columns and was slower than the generic z pass with 8 (8 boxes of 192^3: J form
+// 4.48 against 4.04 ms per step, rho form 4.99 against 4.71; vacuum, the quad kernel
+// ahead, 2.93 against 3.00).
 #define PSATD_REG_Z4(X) X(128) X(192)
 constexpr int z_reg4_tile(int) { return 8; }   // columns per tile
 template <int FORM>

@@ -107,3 +107,33 @@ def test_replayed_direct_captured_and_ordered_launches_agree(built, form, j_cons
         got = run(how)
         for k in want:
             assert np.array_equal(got[k], want[k]), (how, k)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("nsteps", [1, 3])
+def test_chained_launches_in_a_callers_capture(built, nsteps):
+    """A plan on the line kernels, whose launches wait for one another: one push
+    captured by the caller and replayed equals the same pushes launched directly."""
+    import torch
+    from paper_1812_07357_gb300.solver import Plan
+    lay = I.local_layout((40, 32, 24), (2, 1, 1), (5, 4, 3), 4)
+    rng = np.random.default_rng(19)
+    fields = {k: I.scatter_global(rng.standard_normal((24, 32, 40)), lay) for k in O.COMPS}
+    s = torch.cuda.Stream()
+    plan = Plan(lay, (1.0,) * 3, 0.6, precision=32, sources="vacuum", stream=s, no_graph=True)
+    assert plan.fast_boxes == 0
+    with torch.cuda.stream(s):
+        want, got = plan.pack_fields(fields), plan.pack_fields(fields)
+        for _ in range(3):
+            plan.push(want, None, nsteps)
+        plan.sync()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            plan.push(got, None, nsteps)
+        for _ in range(3):
+            g.replay()
+    plan.sync()
+    torch.cuda.synchronize()
+    for k in O.COMPS:
+        assert torch.equal(want[k], got[k]), k
+    plan.close()
