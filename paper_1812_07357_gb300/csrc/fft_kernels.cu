@@ -149,6 +149,19 @@ void z_threads_for(LineCfg& c, int prec, int form, int nft, const std::vector<Ax
   if (cost(96) < 0.97 * cost(128)) c.threads = 96;
 }
 
+// Whether the z pass may start while the y pass drains (kChained).  Its early
+// blocks go wherever room is, so with more than one tile per SM but fewer than
+// the blocks an SM holds (registers: 3, 2 with radices above 16; shared memory)
+// they stack on the SMs that drain first and leave others idle, which the FP64
+// pipe does not hide: one step of a 64^3 box, vacuum (264 tiles) 292 us chained, 248
+// not; 48^3 132, 118; 32 x 32 x 256 314, 257.  With fewer or more tiles it gains: 16^3 33.1
+// against 34.9, 64^3 rho form (528) 329, 332.  FP32 is the same either way.
+int z_chains(int prec, const LineCfg& c, int64_t tiles, int sms) {
+  if (prec == 32 || tiles <= sms) return 1;
+  const int hold = c.cls ? 2 : 3, fit = 227 * 1024 / (c.smem + 1024);
+  return (tiles + sms - 1) / sms >= (hold < fit ? hold : fit);
+}
+
 // Columns per z tile (a power of two, its logarithm in c.lg) and the shared
 // memory of the longest line n2_max: the widest tile of at most 128-byte rows
 // that leaves room for the blocks an SM can hold (FP32 two of 256 threads: two

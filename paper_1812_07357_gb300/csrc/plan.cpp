@@ -420,6 +420,7 @@ struct psatd_plan {
   int64_t field_total = 0;  // elements per field buffer
   int64_t spec_total = 0;   // complex elements per spectrum slot
   bool chain = false;   // every pass of a step is one launch of a line kernel (kChained in direct launches)
+  bool chain_z = true;  // ... the generic z pass too
   LineCfg cfg_x, cfg_y, cfg_z, cfg_zonly;   // generic kernels: launches that cover every box
   int smem_pf = 0, smem_pi = 0, smem_zf = 0;
   int buf_pf = 0, buf_pi = 0, rows_pi = 0;     // complex elements per plane buffer
@@ -1140,6 +1141,7 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
   {
     // one launch per pass, each of a line kernel (register z kernels do not wait)
     P->chain = P->fast_boxes == 0 && P->grp_zreg.empty();
+    P->chain_z = z_chains(P->prec, P->cfg_z, (int64_t)P->g_zcols.size(), P->sms);
   }
   // ---- device memory
   CK(P, upload(P, P->hboxes, &P->d_boxes));
@@ -1831,6 +1833,7 @@ static psatd_status z_step(psatd_plan* P, const DevPlan& D0, cudaStream_t st, in
     ++launches;
   }
   if (!P->g_zcols.empty()) {
+    D = in_pass(P, D0, chain && P->chain_z, *launches_out + launches, false);
     CK(P, timed(P, 2, st, [&] {
          return launch_z_update(P->prec, P->form, D, P->d_ws, S, P->d_g_zcols, (int64_t)P->g_zcols.size(), P->cfg_z,
                                 NFT, st);

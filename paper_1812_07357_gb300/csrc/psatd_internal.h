@@ -225,6 +225,7 @@ int line_lg(int prec, const std::vector<std::pair<AxisPlan, int64_t>>& lines, in
 void z_threads_for(LineCfg& c, int prec, int form, int nft, const std::vector<AxisPlan>& axes, int64_t tiles,
                    int sms);
 void line_cover(LineCfg& c, int prec, const AxisPlan& a, bool rows);
+int z_chains(int prec, const LineCfg& c, int64_t tiles, int sms);
 void z_cover(LineCfg& c, int prec, int form, int n2_max, int64_t columns, int widest, int sms, int optin);
 
 // ---- exchange (exchange.cu) -------------------------------------------------
