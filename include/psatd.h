@@ -460,8 +460,9 @@ int32_t psatd_plan_deferred_exchange(const psatd_plan* plan);
  *   PSATD_TUNE_Z_TILE        most mx columns per tile of the shared-memory
  *                            plane family's and the generic z pass (1 .. 8 in
  *                            FP32, 1 .. 4 in FP64; the generic pass takes the
- *                            power of two below, at least 2 in FP32; default:
- *                            what the kernel chooses).
+ *                            power of two from there up, at least 2 in FP32;
+ *                            default: what the kernel chooses).  FP32 boxes of
+ *                            z length 128 or 192 with sources do not follow it.
  *   PSATD_TUNE_HOST_COPY     (runtime) psatd_push_host's copies: 1 (default)
  *                            = a copy kernel on the SMs reading and writing
  *                            the host buffers through their device mapping

@@ -170,7 +170,7 @@ int z_chains(int prec, const LineCfg& c, int64_t tiles, int sms) {
 // 0.93 against 0.98 with two wider ones) and gives the `columns` columns of the
 // launch a tile per SM (64^3, 10 slots: 264 tiles of 8 columns run at once, 528
 // of 4 columns took two waves, 16.5 us against 12); `widest` > 0: no wider than
-// that.
+// the power of two from there up.
 void z_cover(LineCfg& c, int prec, int form, int n2_max, int64_t columns, int widest, int sms, int optin) {
   const int csz = prec == 32 ? 8 : 16, ns = spec_slots(form);
   const int lo = prec == 32 ? 2 : 1, hi = prec == 32 ? 4 : 3;   // log2 of the narrowest and widest tile
@@ -178,7 +178,7 @@ void z_cover(LineCfg& c, int prec, int form, int n2_max, int64_t columns, int wi
   auto bytes = [&](int lg) { return ns * z_slot_pitch(csz, n2_max, 1 << lg) * csz; };
   int lg = hi;
   while (lg > lo && (bytes(lg) > budget || (columns >> lg) < sms)) --lg;
-  while (lg > lo - 1 && (bytes(lg) > optin || (widest > 0 && (1 << lg) > widest))) --lg;
+  while (lg > lo - 1 && (bytes(lg) > optin || (widest > 0 && (1 << lg) >= 2 * widest))) --lg;
   c.lg = lg;
   c.smem = bytes(lg);
 }

@@ -432,6 +432,7 @@ struct psatd_plan {
   int pen_rows_kb = 64;                        // kept for psatd_plan_tuning; no kernel uses it
   int host_copy = 1;                           // host path: 1 = SM copy kernel on mapped memory, 0 = copy engines
   int z_tile = 0;                              // plane/pencil z tile columns (0: the kernel maximum)
+  bool z_tile_used = false;                    // a z pass of the plan follows it
   // absorbing layers (form kPml): the description, boxes with layer cells,
   // damping table, stored split parts and their per-step increments
   psatd_pml pml{};
@@ -860,7 +861,7 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
   std::vector<int> zgen;
   auto z_boxes = [&](int bi, bool family) {
     const psatd_box& b = P->boxes[bi];
-    if (P->prec == 32 && family) P->pen_reg_z_used = true;
+    if (P->prec == 32 && family && !z_reg_yields(P->form, b.n[2])) P->pen_reg_z_used = true;
     if (P->prec == 32 && family && P->pen_reg_z && z_reg_ok(P->form, b.n[2]) && z_reg_smem(P->form, b.n[2]) <= optin &&
         z_reg_multi_smem(P->form) <= optin) {
       const int L = b.n[0] / 2, n1 = b.n[1], rt = z_reg_tile_width(P->form, b.n[2]);
@@ -967,7 +968,13 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
     zcolumns = INT64_MAX;
     for (const psatd_box& b : P->boxes) zlongest = std::max(zlongest, b.n[2]);
   }
-  z_cover(P->cfg_z, P->prec, P->form, zlongest, zcolumns, P->z_tile, P->sms, optin);
+  // (boxes whose z length had a register z kernel with tiles of its own take no
+  // part in the tile knob)
+  const bool yields_only = P->prec == 32 && !zgen.empty() &&
+                           std::all_of(zgen.begin(), zgen.end(),
+                                       [&](int bi) { return z_reg_yields(P->form, P->boxes[bi].n[2]) != 0; });
+  P->z_tile_used = P->pen_boxes || (P->fast_boxes && !(yields_only && P->zfast.empty()));
+  z_cover(P->cfg_z, P->prec, P->form, zlongest, zcolumns, yields_only ? 0 : P->z_tile, P->sms, optin);
   {
     std::vector<AxisPlan> axes;
     for (int bi : zgen) axes.push_back(P->hshapes[P->hboxes[bi].shape].az);
@@ -2497,7 +2504,7 @@ int32_t psatd_plan_tuning(const psatd_plan* P, int32_t knob) {
     case PSATD_TUNE_Z_ONE_LAUNCH:
       return P->zreg_multi ? P->z_one_launch : -1;
     case PSATD_TUNE_Z_TILE:
-      return (P->pen_boxes || (P->fast_boxes && !P->reg_z))
+      return P->z_tile_used && (P->pen_boxes || !P->reg_z)
                  ? (P->z_tile > 0 ? std::min(P->z_tile, fast_tile(P->prec)) : fast_tile(P->prec))
                  : -1;
     default:

@@ -32,3 +32,29 @@ def test_autotuner_measures_no_unused_knob():
     measure = T.gpu_measure(I.global_layout((64, 64, 64), 8), (1.0,) * 3, 0.5, precision=64)
     _, used = measure("pencil", {"pencil_rows_kb": 32})
     assert "z_tile" in used and "pencil_rows_kb" not in used
+
+
+@pytest.mark.parametrize("n,form,follows", [((128, 128, 128), "rho", False), ((96, 96, 192), "J", False),
+                                            ((128, 128, 160), "rho", True)])
+def test_z_tile_of_long_z_lines_with_sources(n, form, follows):
+    """FP32 boxes on the register planes with sources: z lengths 128 and 192 keep
+    their own tiles whatever z_tile and pencil_reg_z say, so neither is reported; other
+    lengths follow them.  No result depends on it."""
+    import torch
+    from paper_1812_07357_gb300.solver import Plan
+    out = []
+    for tuning in (None, {"z_tile": 1}, {"z_tile": 3}):
+        plan = Plan(I.global_layout(n, 8), (1.0,) * 3, 0.5, precision=32, sources=form, tuning=tuning)
+        assert plan.fast_boxes == 1
+        assert ("z_tile" in plan.tuning()) == follows
+        assert ("pencil_reg_z" in plan.tuning()) == follows
+        g = torch.Generator(device="cuda").manual_seed(3)
+        f = {k: torch.randn(plan.field_elems, device="cuda", generator=g)
+             for k in ("Ex", "Ey", "Ez", "Bx", "By", "Bz", "Jx", "Jy", "Jz", "rho")}
+        s = {k: f[k] for k in ("Jx", "Jy", "Jz")}
+        s["rho"] = f["rho"] if form == "rho" else None
+        plan.push(f, s, 2)
+        plan.sync()
+        out.append(torch.cat([f[k] for k in ("Ex", "By")]))
+        plan.close()
+    assert torch.equal(out[0], out[1]) and torch.equal(out[0], out[2])
