@@ -21,7 +21,8 @@ BUILD = os.path.join(PKG, "_build")
 
 SOURCES = ["plan.cpp", "tables.cu", "fft_kernels.cu", "any_part_0.cu", "any_part_1.cu",
            "any_part_2.cu", "any_part_3.cu", "fast_kernels.cu", "reg_kernels.cu", "reg_planes_0.cu",
-           "reg_planes_1.cu", "reg_planes_2.cu", "reg_planes_3.cu", "exchange.cu", "static_push.cu"]
+           "reg_planes_1.cu", "reg_planes_2.cu", "reg_planes_3.cu", "reg_many_0.cu", "reg_many_1.cu",
+           "reg_many_2.cu", "reg_many_3.cu", "reg_many_z.cu", "exchange.cu", "static_push.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

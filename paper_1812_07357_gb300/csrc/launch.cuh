@@ -7,9 +7,10 @@
 //              (grid_order).  For a launch whose predecessor is a single
 //              launch of the same call, so that its end is the end of all work
 //              before it.
+//   kLeads     ordinary, and the launches after it run beside it: the first launch
+//              of a pass over boxes of several plane shapes or z lengths.
 //   kBeside    starts while the launch before it drains and computes beside it:
-//              for the second and later launches of one pass over different
-//              boxes, the first of which is kOrdinary.  Its grid has one block (or
+//              the later launches of such a pass.  Its grid has one block (or
 //              cluster) more than it has work, which only waits for that launch
 //              to finish (grid_join), so the end of each launch of the pass
 //              implies the end of the one before it.  The launch after the pass is
@@ -17,14 +18,18 @@
 //              only full edge into the next pass comes from the pass's last
 //              launch (a stream would wait for all of them).  It always ends: a
 //              launch starts beside another only when every block of that one
-//              has started.  A block of its own, tested for behind the loads of
-//              the job: 128 boxes of 96^3 2.864 ms per step, against 2.860
-//              without any of it, 2.870 with the test first and 2.909 with a
-//              wait of block 0 at the end of every kernel, which changed their code.
+//              has started.
 //
 // Every kernel here lets its successor start as soon as all its own blocks have
 // (grid_release), so a successor's blocks only take the room that the last
 // wave leaves.
+//
+// The register kernels have instantiations of their own for kLeads and kBeside
+// (MANY): the release alone changed the code of every launch that has no
+// successor beside it.  Steps replayed from graphs, without it / with it / with a
+// join tested behind the loads of the job: 8 boxes of 48^3 rho form 60.3 / 61.7 /
+// 61.9 us, 128 boxes of 96^3 2.832 / 2.836 / 2.839 ms.  The join is a block of its own
+// because a wait of block 0 at the end of every kernel took 2.909.
 //
 // Chained are the line kernels (any_lines.cuh, any_z.cuh, the exchange) of calls
 // that launch directly: a PIC cycle of a 64^3 box 71 -> 62 us, forward + inverse
@@ -57,6 +62,7 @@ __device__ __forceinline__ void grid_join() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 // The grid of a launch of `blocks` blocks per y index, and the extra ones when kBeside.
+inline bool order_of_many(int order) { return order == kLeads || order == kBeside; }
 inline dim3 ordered_grid(int order, unsigned blocks, unsigned y, unsigned n = 1) {
   return dim3(blocks + (order == kBeside ? n : 0u), y);
 }
@@ -73,7 +79,7 @@ cudaError_t launch_ordered(int order, void (*kernel)(P...), dim3 grid, int threa
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
   c.attrs = &attr;
-  c.numAttrs = order == kOrdinary ? 0 : 1;
+  c.numAttrs = order == kChained || order == kBeside ? 1 : 0;
   return cudaLaunchKernelEx(&c, kernel, P(args)...);
 }
 

@@ -1241,7 +1241,8 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
   for (const LineCfg* c : {&P->cfg_x, &P->cfg_y, &P->cfg_zonly, &P->cfg_z}) classes |= 1 << c->cls;
   CK(P, configure_kernels(P->prec, optin, classes));
   CK(P, configure_fast_kernels(P->prec, optin));
-  if (P->prec == 32) CK(P, configure_reg_kernels(optin));
+  if (P->prec == 32)
+    CK(P, configure_reg_kernels(optin, P->grp_pf.size() > 1 || P->grp_pi.size() > 1 || P->grp_zreg.size() > 1));
   if (P->fast_boxes) {
     int sms = 0, occ_f = 0, occ_i = 0;
     CK(P, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -1699,11 +1700,17 @@ psatd_status psatd_guard_exchange(psatd_plan* P, const psatd_fields* f, const ps
 
 // Orders of the launches of one call (launch.cuh): `chain` (a plan's chain
 // flag, never with per-kernel timing) makes every launch but the call's first
-// kChained; the later launches of a pass over several groups are kBeside the
-// first.  `before`: launches of this call so far.
-static DevPlan in_pass(const psatd_plan* P, const DevPlan& D, bool chain, int64_t before, bool later) {
+// kChained.  `before`: launches of this call so far.
+static DevPlan in_pass(const psatd_plan* P, const DevPlan& D, bool chain, int64_t before) {
   DevPlan d = D;
-  d.order = later && !P->timing ? kBeside : chain && before > 0 ? kChained : kOrdinary;
+  d.order = chain && before > 0 ? kChained : kOrdinary;
+  return d;
+}
+
+// Launch i of the n of a pass over several groups of boxes (register kernels).
+static DevPlan of_many(const psatd_plan* P, const DevPlan& D, size_t i, size_t n) {
+  DevPlan d = D;
+  d.order = n == 1 || P->timing ? kOrdinary : i ? kBeside : kLeads;
   return d;
 }
 
@@ -1713,12 +1720,12 @@ static psatd_status forward_xy(psatd_plan* P, const DevPlan& D0, const FieldPtrs
                                cudaStream_t st, int64_t* launches_out, bool gather = false, bool chain = false) {
   const int64_t S = P->spec_total;
   int64_t launches = 0;
-  DevPlan D = in_pass(P, D0, chain, *launches_out, false);
+  DevPlan D = in_pass(P, D0, chain, *launches_out);
   // fast boxes: one plane kernel; generic and pencil boxes: x rows, y columns
   if (!P->grp_pf.empty()) {
     // one launch per register plane shape; the gather tables are indexed by plane_fwd position
     for (const auto& g : P->grp_pf) {
-      D = in_pass(P, D0, chain, *launches_out + launches, &g != &P->grp_pf.front());
+      D = of_many(P, D0, &g - P->grp_pf.data(), P->grp_pf.size());
       if (g.code < 0) {
         CK(P, timed(P, 0, st, [&] {
              return launch_plane_fwd(P->prec, D, fp, nf, spec, S, P->d_plane_fwd + g.start, g.count, P->buf_pf,
@@ -1743,12 +1750,12 @@ static psatd_status forward_xy(psatd_plan* P, const DevPlan& D0, const FieldPtrs
     ++launches;
   }
   if (P->g_nrows) {
-    D = in_pass(P, D0, chain, *launches_out + launches, false);
+    D = in_pass(P, D0, chain, *launches_out + launches);
     CK(P, timed(P, 0, st, [&] {
          return launch_fwd_x(P->prec, D, fp, nf, spec, S, P->d_rows_all, P->g_nrows, P->cfg_x,
                              gather && !P->ggrid.empty() ? P->d_ggrid : nullptr, fields_out(P->form), st);
        }));
-    D = in_pass(P, D0, chain, *launches_out + launches + 1, false);
+    D = in_pass(P, D0, chain, *launches_out + launches + 1);
     CK(P, timed(P, 1, st, [&] {
          return launch_col(P->prec, -1, 1, D, spec, S, nf, P->d_ycols_all, P->g_nycols, P->cfg_y, st);
        }));
@@ -1807,7 +1814,7 @@ static psatd_status z_step(psatd_plan* P, const DevPlan& D0, cudaStream_t st, in
   const int NFT = step_slots(P);
   const int64_t S = P->spec_total;
   int64_t launches = 0;
-  DevPlan D = in_pass(P, D0, chain, *launches_out, false);
+  DevPlan D = in_pass(P, D0, chain, *launches_out);
   const bool one_launch = P->z_one_launch && P->zreg_multi;
   if (one_launch) {
     // every register-z length in one persistent launch, 2 CTAs per SM
@@ -1817,15 +1824,16 @@ static psatd_status z_step(psatd_plan* P, const DevPlan& D0, cudaStream_t st, in
        }));
     ++launches;
   }
-  for (const auto& g : one_launch ? std::vector<psatd_plan::Group>() : P->grp_zreg) {
-    D = in_pass(P, D0, chain, *launches_out + launches, launches > 0);
+  for (size_t i = 0; !one_launch && i < P->grp_zreg.size(); ++i) {
+    const auto& g = P->grp_zreg[i];
+    D = of_many(P, D0, i, P->grp_zreg.size());
     CK(P, timed(P, 2, st, [&] {
          return launch_z_reg(P->form, D, P->d_ws, S, P->d_zpen_reg + g.start, g.count, g.code, 0, NFT, P->z_prefetch,
                              st);
        }));
     ++launches;
   }
-  D = in_pass(P, D0, chain, *launches_out + launches, false);
+  D = in_pass(P, D0, chain, *launches_out + launches);
   if (!P->zfast.empty() && P->reg_z) {
     CK(P, timed(P, 2, st, [&] {
          return launch_z_reg(P->form, D, P->d_ws, S, P->d_zfast, (int64_t)P->zfast.size(), P->reg_z, P->reg_zst,
@@ -1840,7 +1848,7 @@ static psatd_status z_step(psatd_plan* P, const DevPlan& D0, cudaStream_t st, in
     ++launches;
   }
   if (!P->g_zcols.empty()) {
-    D = in_pass(P, D0, chain && P->chain_z, *launches_out + launches, false);
+    D = in_pass(P, D0, chain && P->chain_z, *launches_out + launches);
     CK(P, timed(P, 2, st, [&] {
          return launch_z_update(P->prec, P->form, D, P->d_ws, S, P->d_g_zcols, (int64_t)P->g_zcols.size(), P->cfg_z,
                                 NFT, st);
@@ -1860,12 +1868,12 @@ static psatd_status inverse_step(psatd_plan* P, const DevPlan& D0, const FieldPt
                                  cudaStream_t st, int64_t* launches_out, bool guards, bool chain = false) {
   const int64_t S = P->spec_total;
   int64_t launches = 0;
-  DevPlan D = in_pass(P, D0, chain, *launches_out, false);
+  DevPlan D = in_pass(P, D0, chain, *launches_out);
   // S3: inverse y+x, interior cells only
   if (!P->grp_pi.empty()) {
     // one launch per register plane shape; the guard segments are indexed by plane_inv position
     for (const auto& g : P->grp_pi) {
-      D = in_pass(P, D0, chain, *launches_out + launches, &g != &P->grp_pi.front());
+      D = of_many(P, D0, &g - P->grp_pi.data(), P->grp_pi.size());
       if (g.code < 0) {
         CK(P, timed(P, 4, st, [&] {
              return launch_plane_inv(P->prec, D, fp, nout, spec, S, P->d_plane_inv + g.start, g.count, P->buf_pi,
@@ -1891,11 +1899,11 @@ static psatd_status inverse_step(psatd_plan* P, const DevPlan& D0, const FieldPt
     ++launches;
   }
   if (P->g_nrows) {
-    D = in_pass(P, D0, chain, *launches_out + launches, false);
+    D = in_pass(P, D0, chain, *launches_out + launches);
     CK(P, timed(P, 3, st, [&] {
          return launch_col(P->prec, 1, 1, D, spec, S, nout, P->d_g_ycols_int, (int64_t)P->g_ycols_int.size(), P->cfg_y, st);
        }));
-    D = in_pass(P, D0, chain, *launches_out + launches + 1, false);
+    D = in_pass(P, D0, chain, *launches_out + launches + 1);
     CK(P, timed(P, 4, st, [&] {
          return launch_inv_x(P->prec, D, fp, nout, spec, S, P->d_g_rows_int, (int64_t)P->g_rows_int.size(), P->cfg_x, 1, st);
        }));
@@ -1905,7 +1913,7 @@ static psatd_status inverse_step(psatd_plan* P, const DevPlan& D0, const FieldPt
     // absorbing layers, step (2): damp the split parts, rebuild the components
     FieldPtrs parts{};
     for (int q = 0; q < 6; ++q) parts.p[q] = P->pml_parts[q];
-    D = in_pass(P, D0, chain, *launches_out + launches, false);
+    D = in_pass(P, D0, chain, *launches_out + launches);
     CK(P, timed(P, 4, st, [&] {
          return launch_pml_damp(P->prec, D, fp, parts, P->d_pml_boxes, (int)P->pml_boxes.size(), P->d_pml_tab,
                                 P->pml_tab, st);
@@ -1914,7 +1922,7 @@ static psatd_status inverse_step(psatd_plan* P, const DevPlan& D0, const FieldPt
   }
   if (!P->step_tiles.empty() && guards) {
     const int nex = P->form == kPml ? 6 : nout;   // components only, not the increments
-    D = in_pass(P, D0, chain, *launches_out + launches, false);
+    D = in_pass(P, D0, chain, *launches_out + launches);
     CK(P, timed(P, 5, st, [&] {
          return launch_exchange(P->prec, D, fp, nex, P->d_blocks, P->d_step_tiles, (int64_t)P->step_tiles.size(),
                                 st);

@@ -175,7 +175,7 @@ struct alignas(4 * sizeof(T)) Coef4 {
 };
 
 // Order of a launch against the one before it (launch.cuh).
-enum LaunchOrder { kOrdinary = 0, kChained = 1, kBeside = 2 };
+enum LaunchOrder { kOrdinary = 0, kChained = 1, kBeside = 2, kLeads = 3 };
 
 // Device view of a plan, passed by value to every kernel.
 struct DevPlan {
@@ -298,9 +298,12 @@ cudaError_t launch_plane_fwd_reg(int code, const DevPlan& P, const FieldPtrs& f,
 cudaError_t launch_plane_inv_reg(int code, const DevPlan& P, const FieldPtrs& f, int nf, void* spec,
                                  int64_t sstride, const int2* jobs, int64_t nplanes, const int* seg_start,
                                  const GuardSeg* segs, cudaStream_t st);
-cudaError_t configure_reg_kernels(int smem_bytes);
-// the plane shapes are instantiated in four translation units
-// (reg_planes_<part>.cu); each exports its launchers in namespace plane_part<part>
+// many: the instantiations for passes of several launches (kLeads, kBeside) too; a
+// kernel is loaded when its attribute is first set
+cudaError_t configure_reg_kernels(int smem_bytes, bool many);
+// the plane shapes are instantiated in four translation units (reg_planes_<part>.cu,
+// launchers in namespace plane_part<part>), and again for passes of several launches
+// (reg_many_<part>.cu, plane_many<part>), whose modules only plans that have such passes load
 #define PSATD_DECLARE_PLANE_PART(NS)                                                                       \
   namespace NS {                                                                                           \
   cudaError_t launch_fwd(int code, const DevPlan& P, const FieldPtrs& f, int nf, void* spec, int64_t sstride,  \
@@ -315,6 +318,10 @@ PSATD_DECLARE_PLANE_PART(plane_part0)
 PSATD_DECLARE_PLANE_PART(plane_part1)
 PSATD_DECLARE_PLANE_PART(plane_part2)
 PSATD_DECLARE_PLANE_PART(plane_part3)
+PSATD_DECLARE_PLANE_PART(plane_many0)
+PSATD_DECLARE_PLANE_PART(plane_many1)
+PSATD_DECLARE_PLANE_PART(plane_many2)
+PSATD_DECLARE_PLANE_PART(plane_many3)
 #undef PSATD_DECLARE_PLANE_PART
 // register z kernel (FP32, tiles of z_reg_tile_width(form, n2) columns) for z
 // length n2 (thread pairs per column; thread quads for 128 and 192, vacuum form)
@@ -329,6 +336,10 @@ int z_reg_tile_width(int form, int n2);
 // length; 2 * ns * tile <= 64)
 cudaError_t launch_z_fwd_pair(const DevPlan& P, void* spec, int64_t sstride, const ColJob* jobs, int64_t njobs,
                               int n2, int tile, int ns, cudaStream_t st);
+// register z kernels for passes of several launches (reg_many_z.cu)
+cudaError_t launch_z_many(int form, const DevPlan& P, void* spec, int64_t sstride, const ColJob* jobs, int64_t njobs,
+                          int n2, int nft, int pf_dist, cudaStream_t st);
+cudaError_t configure_z_many(int smem_bytes);
 // zst: n1 * (n0/2 + 1) shared by every box of the job list, else 0
 // pf_dist > 0: every CTA first prefetches into L2 the tile of the CTA
 // launched pf_dist blocks after it

@@ -214,14 +214,14 @@ __device__ __forceinline__ void z_reg_tile_job(const DevPlan& P, float2* spec, i
 }
 
 // One CTA per z tile, every box of the launch with z length NZ.
-template <int NZ, int FORM, int ZST>
+template <int NZ, int FORM, int ZST, bool MANY>
 __global__ void __launch_bounds__(z_reg_threads<FORM>(), z_reg_min_blocks<FORM>())
     k_z_reg(DevPlan P, float2* spec, int64_t sstride, const ColJob* __restrict__ jobs, int nft, int njobs,
             int pf_dist) {
-  if (grid_extra(P.order)) return grid_join();
+  if (MANY && grid_extra(P.order)) return grid_join();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const ColJob J = jobs[blockIdx.x];
-  grid_release();
+  if (MANY) grid_release();
   // the tile that a CTA launched about pf_dist blocks later will read: fetched
   // into L2 now, so that its loads hit L2 instead of waiting on HBM
   if (pf_dist > 0 && (int)blockIdx.x + pf_dist < njobs)
@@ -368,14 +368,14 @@ __device__ __forceinline__ void z_reg4_tile_job(const DevPlan& P, float2* spec, 
   }
 }
 
-template <int NZ, int FORM>
+template <int NZ, int FORM, bool MANY>
 __global__ void __launch_bounds__(z_reg4_threads<FORM>(), 2)
     k_z_reg4(DevPlan P, float2* spec, int64_t sstride, const ColJob* __restrict__ jobs, int nft, int njobs,
              int pf_dist) {
-  if (grid_extra(P.order)) return grid_join();
+  if (MANY && grid_extra(P.order)) return grid_join();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const ColJob J = jobs[blockIdx.x];
-  grid_release();
+  if (MANY) grid_release();
   if (pf_dist > 0 && (int)blockIdx.x + pf_dist < njobs)
     prefetch_z_tile<NZ, FORM, z_reg4_threads<FORM>()>(P, spec, sstride, jobs[blockIdx.x + pf_dist]);
   z_reg4_tile_job<NZ, FORM>(P, spec, sstride, J, nft, smem_raw);
@@ -421,6 +421,60 @@ __global__ void __launch_bounds__(64) k_z_fwd_pair(DevPlan P, float2* spec, int6
   }
 }
 }  // namespace
+
+#ifdef PSATD_Z_MANY
+
+cudaError_t launch_z_many(int form, const DevPlan& P, void* spec, int64_t sstride, const ColJob* jobs, int64_t njobs,
+                          int n2, int nft, int pf_dist, cudaStream_t st) {
+  const dim3 grid = ordered_grid(P.order, (unsigned)njobs, 1);
+  const int smem = z_reg_smem(form, n2);
+  float2* s = (float2*)spec;
+#define PSATD_ZF(NZV, F)                                                                                    \
+  launch_ordered(P.order, k_z_reg<NZV, F, 0, true>, grid, z_reg_threads<F>(), smem, st, P, s, sstride, jobs, nft, \
+                 (int)njobs, pf_dist)
+#define PSATD_ZL(NZV)               \
+  if (n2 == NZV) {                  \
+    if (form == kVacuum)            \
+      PSATD_ZF(NZV, kVacuum);       \
+    else if (form == kJForm)        \
+      PSATD_ZF(NZV, kJForm);        \
+    else                            \
+      PSATD_ZF(NZV, kRhoForm);      \
+  }
+  PSATD_REG_Z(PSATD_ZL)
+#undef PSATD_ZL
+#undef PSATD_ZF
+#define PSATD_ZL(NZV)                                                                                            \
+  if (n2 == NZV) {                                                                                              \
+    if (form != kVacuum) return cudaErrorInvalidValue;                                                           \
+    launch_ordered(P.order, k_z_reg4<NZV, kVacuum, true>, grid, z_reg4_threads<kVacuum>(), smem, st, P, s, sstride, \
+                   jobs, nft, (int)njobs, pf_dist);                                                              \
+  }
+  PSATD_REG_Z4(PSATD_ZL)
+#undef PSATD_ZL
+  return cudaGetLastError();
+}
+
+cudaError_t configure_z_many(int smem) {
+  cudaError_t e = cudaSuccess;
+  auto set = [&](const void* k, int bytes) {
+    const cudaError_t r =
+        bytes <= smem ? cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) : cudaSuccess;
+    if (r != cudaSuccess) e = r;
+  };
+#define PSATD_ZA(NZV)                                                          \
+  set((const void*)k_z_reg<NZV, kVacuum, 0, true>, z_reg_smem(kVacuum, NZV));   \
+  set((const void*)k_z_reg<NZV, kJForm, 0, true>, z_reg_smem(kJForm, NZV));     \
+  set((const void*)k_z_reg<NZV, kRhoForm, 0, true>, z_reg_smem(kRhoForm, NZV));
+  PSATD_REG_Z(PSATD_ZA)
+#undef PSATD_ZA
+#define PSATD_ZA(NZV) set((const void*)k_z_reg4<NZV, kVacuum, true>, z_reg_smem(kVacuum, NZV));
+  PSATD_REG_Z4(PSATD_ZA)
+#undef PSATD_ZA
+  return e;
+}
+
+#else
 
 static bool z_reg_quad(int n2) {
 #define PSATD_ZC(NZV) \
@@ -470,10 +524,11 @@ constexpr int kRegZst = 96 * 49;
 cudaError_t launch_z_reg(int form, const DevPlan& P, void* spec, int64_t sstride, const ColJob* jobs,
                          int64_t njobs, int n2, int zst, int nft, int pf_dist, cudaStream_t st) {
   if (njobs <= 0) return cudaSuccess;
-  const dim3 grid = ordered_grid(P.order, (unsigned)njobs, 1);
+  if (order_of_many(P.order)) return launch_z_many(form, P, spec, sstride, jobs, njobs, n2, nft, pf_dist, st);
+  const dim3 grid((unsigned)njobs);
   const int smem = z_reg_smem(form, n2);
 #define PSATD_ZF(NZV, F, ZS)                                                                      \
-  launch_ordered(P.order, k_z_reg<NZV, F, ZS>, grid, z_reg_threads<F>(), smem, st, P, (float2*)spec, \
+  launch_ordered(P.order, k_z_reg<NZV, F, ZS, false>, grid, z_reg_threads<F>(), smem, st, P, (float2*)spec, \
                  sstride, jobs, nft, (int)njobs, pf_dist)
 #define PSATD_ZL(NZV)                                                    \
   if (n2 == NZV) {                                                      \
@@ -500,7 +555,7 @@ cudaError_t launch_z_reg(int form, const DevPlan& P, void* spec, int64_t sstride
 #define PSATD_ZL(NZV)                                                                                     \
   if (n2 == NZV) {                                                                                       \
     if (form != kVacuum) return cudaErrorInvalidValue;                                                    \
-    launch_ordered(P.order, k_z_reg4<NZV, kVacuum>, grid, z_reg4_threads<kVacuum>(), smem, st, P, (float2*)spec,  \
+    launch_ordered(P.order, k_z_reg4<NZV, kVacuum, false>, grid, z_reg4_threads<kVacuum>(), smem, st, P, (float2*)spec,  \
                    sstride, jobs, nft, (int)njobs, pf_dist);                                              \
   }
   PSATD_REG_Z4(PSATD_ZL)
@@ -574,11 +629,12 @@ static int reg_plane_part(int code) {
 cudaError_t launch_plane_fwd_reg(int code, const DevPlan& P, const FieldPtrs& f, int nf, void* spec,
                                  int64_t sstride, const int2* jobs, int64_t nplanes, const int* gstart,
                                  const GatherSeg* gsegs, const GatherGrid* ggrid, int ngather, cudaStream_t st) {
+  const bool many = order_of_many(P.order);
   switch (reg_plane_part(code)) {
-    case 0: return plane_part0::launch_fwd(code, P, f, nf, spec, sstride, jobs, nplanes, gstart, gsegs, ggrid, ngather, st);
-    case 1: return plane_part1::launch_fwd(code, P, f, nf, spec, sstride, jobs, nplanes, gstart, gsegs, ggrid, ngather, st);
-    case 2: return plane_part2::launch_fwd(code, P, f, nf, spec, sstride, jobs, nplanes, gstart, gsegs, ggrid, ngather, st);
-    case 3: return plane_part3::launch_fwd(code, P, f, nf, spec, sstride, jobs, nplanes, gstart, gsegs, ggrid, ngather, st);
+    case 0: return (many ? plane_many0::launch_fwd : plane_part0::launch_fwd)(code, P, f, nf, spec, sstride, jobs, nplanes, gstart, gsegs, ggrid, ngather, st);
+    case 1: return (many ? plane_many1::launch_fwd : plane_part1::launch_fwd)(code, P, f, nf, spec, sstride, jobs, nplanes, gstart, gsegs, ggrid, ngather, st);
+    case 2: return (many ? plane_many2::launch_fwd : plane_part2::launch_fwd)(code, P, f, nf, spec, sstride, jobs, nplanes, gstart, gsegs, ggrid, ngather, st);
+    case 3: return (many ? plane_many3::launch_fwd : plane_part3::launch_fwd)(code, P, f, nf, spec, sstride, jobs, nplanes, gstart, gsegs, ggrid, ngather, st);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -586,11 +642,12 @@ cudaError_t launch_plane_fwd_reg(int code, const DevPlan& P, const FieldPtrs& f,
 cudaError_t launch_plane_inv_reg(int code, const DevPlan& P, const FieldPtrs& f, int nf, void* spec,
                                  int64_t sstride, const int2* jobs, int64_t nplanes, const int* seg_start,
                                  const GuardSeg* segs, cudaStream_t st) {
+  const bool many = order_of_many(P.order);
   switch (reg_plane_part(code)) {
-    case 0: return plane_part0::launch_inv(code, P, f, nf, spec, sstride, jobs, nplanes, seg_start, segs, st);
-    case 1: return plane_part1::launch_inv(code, P, f, nf, spec, sstride, jobs, nplanes, seg_start, segs, st);
-    case 2: return plane_part2::launch_inv(code, P, f, nf, spec, sstride, jobs, nplanes, seg_start, segs, st);
-    case 3: return plane_part3::launch_inv(code, P, f, nf, spec, sstride, jobs, nplanes, seg_start, segs, st);
+    case 0: return (many ? plane_many0::launch_inv : plane_part0::launch_inv)(code, P, f, nf, spec, sstride, jobs, nplanes, seg_start, segs, st);
+    case 1: return (many ? plane_many1::launch_inv : plane_part1::launch_inv)(code, P, f, nf, spec, sstride, jobs, nplanes, seg_start, segs, st);
+    case 2: return (many ? plane_many2::launch_inv : plane_part2::launch_inv)(code, P, f, nf, spec, sstride, jobs, nplanes, seg_start, segs, st);
+    case 3: return (many ? plane_many3::launch_inv : plane_part3::launch_inv)(code, P, f, nf, spec, sstride, jobs, nplanes, seg_start, segs, st);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -598,14 +655,18 @@ cudaError_t launch_plane_inv_reg(int code, const DevPlan& P, const FieldPtrs& f,
 // Dynamic shared memory limits of the register kernels: what each launch
 // asks for (the gather table of the forward kernel is static shared memory
 // on top of it); `smem` is the device's opt-in maximum.
-cudaError_t configure_reg_kernels(int smem) {
+cudaError_t configure_reg_kernels(int smem, bool many) {
   cudaError_t e = cudaSuccess;
   for (cudaError_t r : {plane_part0::configure(smem), plane_part1::configure(smem), plane_part2::configure(smem),
                         plane_part3::configure(smem)})
     if (r != cudaSuccess) e = r;
+  if (many)
+    for (cudaError_t r : {plane_many0::configure(smem), plane_many1::configure(smem), plane_many2::configure(smem),
+                          plane_many3::configure(smem), configure_z_many(smem)})
+      if (r != cudaSuccess) e = r;
 #define PSATD_ZA(NZV, F, ZS)                                                                      \
   if (z_reg_smem(F, NZV) <= smem) {                                                               \
-    const cudaError_t r = cudaFuncSetAttribute(k_z_reg<NZV, F, ZS>,                               \
+    const cudaError_t r = cudaFuncSetAttribute(k_z_reg<NZV, F, ZS, false>,                               \
                                                cudaFuncAttributeMaxDynamicSharedMemorySize,       \
                                                z_reg_smem(F, NZV));                               \
     if (r != cudaSuccess) e = r;                                                                  \
@@ -623,7 +684,7 @@ cudaError_t configure_reg_kernels(int smem) {
 #define PSATD_ZA(NZV, F)                                                                                  \
   if (z_reg_smem(F, NZV) <= smem) {                                                                       \
     const cudaError_t r =                                                                                 \
-        cudaFuncSetAttribute(k_z_reg4<NZV, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, z_reg_smem(F, NZV)); \
+        cudaFuncSetAttribute(k_z_reg4<NZV, F, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, z_reg_smem(F, NZV)); \
     if (r != cudaSuccess) e = r;                                                                          \
   }
 #define PSATD_ZS(NZV) PSATD_ZA(NZV, kVacuum)
@@ -642,5 +703,7 @@ cudaError_t configure_reg_kernels(int smem) {
 #undef PSATD_ZMA
   return e;
 }
+
+#endif  // PSATD_Z_MANY
 
 }  // namespace psatd

@@ -140,7 +140,7 @@ __device__ __forceinline__ void plane_load(const DevPlan& P, const FieldPtrs& F,
 }
 
 // ---------------------------------------------------------------------------
-template <int L, int NY>
+template <int L, int NY, bool MANY>
 __global__ void __launch_bounds__(reg_plane_threads<L, NY>(), reg_plane_min_blocks<L, NY>())
     k_plane_fwd_reg(DevPlan P, FieldPtrs F, float2* spec, int64_t sstride, const int2* __restrict__ jobs,
                     const int* __restrict__ gstart, const GatherSeg* __restrict__ gsegs,
@@ -150,11 +150,11 @@ __global__ void __launch_bounds__(reg_plane_threads<L, NY>(), reg_plane_min_bloc
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ float2 wsc[NY];   // y transform of the packed real columns
   float* buf = reinterpret_cast<float*>(smem_raw);
-  const bool extra = grid_extra(P.order);
+  const bool extra = MANY && grid_extra(P.order);
   const int2 J = jobs[blockIdx.x - extra];   // an extra block makes no use of it
   const int f = blockIdx.y;
   const BoxDev bx = P.boxes[J.x];
-  grid_release();
+  if (MANY) grid_release();
   if (extra) return grid_join();
   plane_load<N0, NY, NT>(P, F, buf, J, f, bx, gstart, gsegs, ggrid, ngather);
   // x: row r -> half spectrum X[0..L] written back into the same row
@@ -267,7 +267,7 @@ __device__ __forceinline__ void plane_store(const DevPlan& P, const FieldPtrs& F
   }
 }
 
-template <int L, int NY>
+template <int L, int NY, bool MANY>
 __global__ void __launch_bounds__(reg_plane_threads<L, NY>(), reg_plane_min_blocks<L, NY>())
     k_plane_inv_reg(DevPlan P, FieldPtrs F, const float2* spec, int64_t sstride, const int2* __restrict__ jobs,
                     const int* __restrict__ seg_start, const GuardSeg* __restrict__ segs) {
@@ -278,11 +278,11 @@ __global__ void __launch_bounds__(reg_plane_threads<L, NY>(), reg_plane_min_bloc
   // consumed, the interior rows (pitch PF floats): X values, then real cells
   float2* sp = reinterpret_cast<float2*>(smem_raw);
   float* rows = reinterpret_cast<float*>(smem_raw);
-  const bool extra = grid_extra(P.order);
+  const bool extra = MANY && grid_extra(P.order);
   const int2 J = jobs[blockIdx.x - extra];   // an extra block makes no use of it
   const int f = blockIdx.y;
   const BoxDev bx = P.boxes[J.x];
-  grid_release();
+  if (MANY) grid_release();
   if (extra) return grid_join();
   const int ylo = bx.ng_lo[1], yhi = NY - bx.ng_hi[1], ni = yhi - ylo;
   const int xlo = bx.ng_lo[0], nxi = N0 - bx.ng_lo[0] - bx.ng_hi[0];
@@ -414,7 +414,7 @@ __device__ __forceinline__ float2 root_q(int q) {
   return w;
 }
 
-template <int L, int NY>
+template <int L, int NY, bool MANY>
 __global__ void __launch_bounds__(wide_threads<L, NY>(), wide_min_blocks<L, NY>())
     k_plane_fwd_wide(DevPlan P, FieldPtrs F, float2* spec, int64_t sstride, const int2* __restrict__ jobs,
                      const int* __restrict__ gstart, const GatherSeg* __restrict__ gsegs,
@@ -426,11 +426,11 @@ __global__ void __launch_bounds__(wide_threads<L, NY>(), wide_min_blocks<L, NY>(
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* buf = reinterpret_cast<float*>(smem_raw);
   float2* cb = reinterpret_cast<float2*>(smem_raw);
-  const bool extra = grid_extra(P.order);
+  const bool extra = MANY && grid_extra(P.order);
   const int2 J = jobs[blockIdx.x - extra];   // an extra block makes no use of it
   const int f = blockIdx.y;
   const BoxDev bx = P.boxes[J.x];
-  grid_release();
+  if (MANY) grid_release();
   if (extra) return grid_join();
   plane_load<N0, NY, NT>(P, F, buf, J, f, bx, gstart, gsegs, ggrid, ngather);
   const int t = threadIdx.x;
@@ -560,7 +560,7 @@ __global__ void __launch_bounds__(wide_threads<L, NY>(), wide_min_blocks<L, NY>(
   }
 }
 
-template <int L, int NY>
+template <int L, int NY, bool MANY>
 __global__ void __launch_bounds__(wide_threads<L, NY>(), wide_min_blocks<L, NY>())
     k_plane_inv_wide(DevPlan P, FieldPtrs F, const float2* spec, int64_t sstride, const int2* __restrict__ jobs,
                      const int* __restrict__ seg_start, const GuardSeg* __restrict__ segs) {
@@ -574,11 +574,11 @@ __global__ void __launch_bounds__(wide_threads<L, NY>(), wide_min_blocks<L, NY>(
   float2* sp = reinterpret_cast<float2*>(smem_raw);
   float2* cb = reinterpret_cast<float2*>(smem_raw);
   float* rows = reinterpret_cast<float*>(smem_raw);
-  const bool extra = grid_extra(P.order);
+  const bool extra = MANY && grid_extra(P.order);
   const int2 J = jobs[blockIdx.x - extra];   // an extra block makes no use of it
   const int f = blockIdx.y;
   const BoxDev bx = P.boxes[J.x];
-  grid_release();
+  if (MANY) grid_release();
   if (extra) return grid_join();
   const int ylo = bx.ng_lo[1], yhi = NY - bx.ng_hi[1], ni = yhi - ylo;
   const int xlo = bx.ng_lo[0], nxi = N0 - bx.ng_lo[0] - bx.ng_hi[0];
@@ -813,12 +813,12 @@ __device__ __forceinline__ void plane_load_rows(const FieldPtrs& F, float* buf, 
   __syncthreads();
 }
 
-template <int L, int NY>
+template <int L, int NY, bool MANY>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split_threads<L, NY>(), 2)
     k_plane_fwd_split(DevPlan P, FieldPtrs F, float2* spec, int64_t sstride, const int2* __restrict__ jobs,
                       const int* __restrict__ gstart, const GatherSeg* __restrict__ gsegs,
                       const GatherGrid* __restrict__ ggrid, int ngather) {
-  if (grid_extra(P.order, 2)) return grid_join();
+  if (MANY && grid_extra(P.order, 2)) return grid_join();
   constexpr int N0 = 2 * L, HX = L + 1, PF = row_pitch(N0), PC = PF / 2;
   constexpr int GX = wide_gx<L, NY>(), GY = wide_gy<L, NY>(), NT = split_threads<L, NY>();
   constexpr int LX = L / GX, LY = NY / GY, LXP = GX > 1 ? LX + 1 : LX;
@@ -835,7 +835,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split_threads<L, NY>
   const int2 J = jobs[pj];
   const int f = blockIdx.y;
   const BoxDev bx = P.boxes[J.x];
-  grid_release();
+  if (MANY) grid_release();
   plane_load_rows<N0, NY, NT, NH>(F, buf, J, f, bx, pj, h * NH, gstart, gsegs, ggrid, ngather);
   const int t = threadIdx.x;
   // x, stage 1 on the CTA's rows (as k_plane_fwd_wide)
@@ -959,10 +959,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split_threads<L, NY>
 }  // namespace
 
 // ---------------------------------------------------------------------------
-// The launchers of one part (PSATD_PLANE_PART): every shape of the part, by code.
+// The launchers of one part (PSATD_PLANE_PART), namespace PSATD_PLANE_NS: every shape
+// of the part, by code, with kernels for single launches or for the launches of
+// a pass over several shapes (PSATD_PLANE_MANY).
 #ifdef PSATD_PLANE_PART
-#define PSATD_PART_CAT2(a, b) a##b
-#define PSATD_PART_CAT(a, b) PSATD_PART_CAT2(a, b)
 namespace {
 
 // bytes of dynamic shared memory: the real plane with its row pitch (forward);
@@ -983,13 +983,13 @@ bool plane_fwd_shape(int code, dim3 grid, const DevPlan& P, const FieldPtrs& f, 
   if constexpr (PART == PSATD_PLANE_PART) {
     if (code != CODE) return false;
     if constexpr (plane_is_split<L, NY>())
-      launch_ordered(P.order, k_plane_fwd_split<L, NY>, ordered_grid(P.order, 2 * grid.x, grid.y, 2),
+      launch_ordered(P.order, k_plane_fwd_split<L, NY, PSATD_PLANE_MANY>, ordered_grid(P.order, 2 * grid.x, grid.y, 2),
                      split_threads<L, NY>(), split_smem<L, NY>(), st, P, f, (float2*)spec, sstride, jobs, gstart, gsegs, ggrid, ngather);
     else if constexpr (plane_is_wide<L, NY>())
-      launch_ordered(P.order, k_plane_fwd_wide<L, NY>, ordered_grid(P.order, grid.x, grid.y),
+      launch_ordered(P.order, k_plane_fwd_wide<L, NY, PSATD_PLANE_MANY>, ordered_grid(P.order, grid.x, grid.y),
                      wide_threads<L, NY>(), plane_fwd_bytes<L, NY>(), st, P, f, (float2*)spec, sstride, jobs, gstart, gsegs, ggrid, ngather);
     else
-      launch_ordered(P.order, k_plane_fwd_reg<L, NY>, ordered_grid(P.order, grid.x, grid.y),
+      launch_ordered(P.order, k_plane_fwd_reg<L, NY, PSATD_PLANE_MANY>, ordered_grid(P.order, grid.x, grid.y),
                      reg_plane_threads<L, NY>(), plane_fwd_bytes<L, NY>(), st, P, f, (float2*)spec, sstride, jobs, gstart, gsegs, ggrid, ngather);
     return true;
   } else {
@@ -1003,10 +1003,10 @@ bool plane_inv_shape(int code, dim3 grid, const DevPlan& P, const FieldPtrs& f, 
   if constexpr (PART == PSATD_PLANE_PART) {
     if (code != CODE) return false;
     if constexpr (plane_is_wide<L, NY>())
-      launch_ordered(P.order, k_plane_inv_wide<L, NY>, ordered_grid(P.order, grid.x, grid.y),
+      launch_ordered(P.order, k_plane_inv_wide<L, NY, PSATD_PLANE_MANY>, ordered_grid(P.order, grid.x, grid.y),
                      wide_threads<L, NY>(), plane_inv_bytes<L, NY>(), st, P, f, (const float2*)spec, sstride, jobs, seg_start, segs);
     else
-      launch_ordered(P.order, k_plane_inv_reg<L, NY>, ordered_grid(P.order, grid.x, grid.y),
+      launch_ordered(P.order, k_plane_inv_reg<L, NY, PSATD_PLANE_MANY>, ordered_grid(P.order, grid.x, grid.y),
                      reg_plane_threads<L, NY>(), plane_inv_bytes<L, NY>(), st, P, f, (const float2*)spec, sstride, jobs, seg_start, segs);
     return true;
   } else {
@@ -1020,26 +1020,26 @@ void plane_configure_shape(int smem, cudaError_t* e) {
     if (plane_fwd_bytes<L, NY>() > smem || plane_inv_bytes<L, NY>() > smem) return;
     cudaError_t r, r2;
     if constexpr (plane_is_split<L, NY>()) {
-      r = cudaFuncSetAttribute(k_plane_fwd_split<L, NY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      r = cudaFuncSetAttribute(k_plane_fwd_split<L, NY, PSATD_PLANE_MANY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                split_smem<L, NY>());
-      r2 = cudaFuncSetAttribute(k_plane_inv_wide<L, NY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      r2 = cudaFuncSetAttribute(k_plane_inv_wide<L, NY, PSATD_PLANE_MANY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 plane_inv_bytes<L, NY>());
     } else if constexpr (plane_is_wide<L, NY>()) {
-      r = cudaFuncSetAttribute(k_plane_fwd_wide<L, NY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      r = cudaFuncSetAttribute(k_plane_fwd_wide<L, NY, PSATD_PLANE_MANY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                plane_fwd_bytes<L, NY>());
-      r2 = cudaFuncSetAttribute(k_plane_inv_wide<L, NY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      r2 = cudaFuncSetAttribute(k_plane_inv_wide<L, NY, PSATD_PLANE_MANY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 plane_inv_bytes<L, NY>());
     } else {
-      r = cudaFuncSetAttribute(k_plane_fwd_reg<L, NY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      r = cudaFuncSetAttribute(k_plane_fwd_reg<L, NY, PSATD_PLANE_MANY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                plane_fwd_bytes<L, NY>());
-      r2 = cudaFuncSetAttribute(k_plane_inv_reg<L, NY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      r2 = cudaFuncSetAttribute(k_plane_inv_reg<L, NY, PSATD_PLANE_MANY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 plane_inv_bytes<L, NY>());
       // the whole unified L1 as shared memory: room for every CTA the
       // register budget allows
       if (r == cudaSuccess)
-        r = cudaFuncSetAttribute(k_plane_fwd_reg<L, NY>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        r = cudaFuncSetAttribute(k_plane_fwd_reg<L, NY, PSATD_PLANE_MANY>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
       if (r2 == cudaSuccess)
-        r2 = cudaFuncSetAttribute(k_plane_inv_reg<L, NY>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        r2 = cudaFuncSetAttribute(k_plane_inv_reg<L, NY, PSATD_PLANE_MANY>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     }
     if (r != cudaSuccess) *e = r;
     if (r2 != cudaSuccess) *e = r2;
@@ -1048,7 +1048,7 @@ void plane_configure_shape(int smem, cudaError_t* e) {
 
 }  // namespace
 
-namespace PSATD_PART_CAT(plane_part, PSATD_PLANE_PART) {
+namespace PSATD_PLANE_NS {
 
 cudaError_t launch_fwd(int code, const DevPlan& P, const FieldPtrs& f, int nf, void* spec, int64_t sstride,
                        const int2* jobs, int64_t nplanes, const int* gstart, const GatherSeg* gsegs,
@@ -1082,9 +1082,7 @@ cudaError_t configure(int smem) {
   return e;
 }
 
-}  // namespace plane_part<PSATD_PLANE_PART>
-#undef PSATD_PART_CAT
-#undef PSATD_PART_CAT2
+}  // namespace PSATD_PLANE_NS
 #endif  // PSATD_PLANE_PART
 
 }  // namespace psatd
