@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(line_threads<T, CLS>(), sizeof(T) == 4 && !CLS
   if constexpr (sizeof(T) == 4) {
     // lanes along the row: every thread merges its own samples from HBM (both
     // ends of a pair, the other end from L1) and stores its outputs to HBM
-    const T scale = bx.scale32;
+    const T scale = sh.scale32;
     const int pitch = row_line_pitch(sh.ax), p2 = l.r2 | 1;
     {
       const int r = line_div(threadIdx.x, line_magic(l.r2)), n2 = threadIdx.x - r * l.r2;
@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(line_threads<T, CLS>(), sizeof(T) == 4 && !CLS
         }
       });
   } else {
-    const T scale = bx.scale64;
+    const T scale = sh.scale64;
     const int PX = hx | 1;
     const unsigned mh = line_magic(hx);
     for (int e = threadIdx.x; e < J.nr * hx; e += blockDim.x) cp_async(sm + e + line_div(e, mh) * (PX - hx), in + e);

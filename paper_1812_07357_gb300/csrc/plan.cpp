@@ -759,6 +759,8 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
     s.L = b.n[0] / 2;
     s.hx = s.L + 1;
     s.p = b.order_p;
+    s.scale64 = 1.0 / ((double)b.n[0] * b.n[1] * b.n[2]);
+    s.scale32 = (float)s.scale64;
     if (!line_plan(s.L, s.ax, P->prec, true) || !line_plan(b.n[1], s.ay, P->prec, false) ||
         !line_plan(b.n[2], s.az, P->prec, false))
       return fail(nullptr, PSATD_ERR_UNSUPPORTED_SIZE, "no radix schedule");
@@ -816,8 +818,6 @@ psatd_status build(psatd_plan* P, cudaStream_t st) {
     gplane += b.n[2];
     x.foff = foff;
     x.soff = soff;
-    x.scale64 = 1.0 / ((double)b.n[0] * b.n[1] * b.n[2]);
-    x.scale32 = (float)x.scale64;
     foff += align_up((int64_t)b.n[0] * b.n[1] * b.n[2], 64);
     soff += align_up((int64_t)(b.n[0] / 2 + 1) * b.n[1] * b.n[2], 32);
     P->hboxes.push_back(x);

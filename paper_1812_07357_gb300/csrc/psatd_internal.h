@@ -60,6 +60,9 @@ struct ShapeDev {
   int32_t fx, fy, fz;             // fast-length codes of L, n1, n2 (-1: not a fast length)
   int32_t px, py, pz;             // pencil-length codes of L, n1, n2 (-1: none)
   int32_t lp, hp;                 // smem row pitches (complex) of the fast plane kernels
+  double scale64;                 // 1 / (n0 n1 n2), the inverse transform's factor (not in BoxDev, which the
+  float scale32;                  // guard loops load per rectangle) ... rounded once
+  int32_t pad;
 };
 
 // Lengths with a two-pass register FFT, N = R1 * R2: X(code, N, R1, R2).
@@ -103,9 +106,6 @@ struct BoxDev {
   int32_t yoff;                   // global index of the box's spectrum row my = 0 (rows of a distributed group)
   int64_t foff;                   // element offset in every field buffer
   int64_t soff;                   // complex-element offset in every spectrum slot
-  double scale64;                 // 1 / (n0 n1 n2), the inverse transform's factor
-  float scale32;                  // ... rounded once
-  int32_t pad;
 };
 
 // rows r0 .. r0+nr-1 of one box, row r = y + n1*z (x-axis passes)

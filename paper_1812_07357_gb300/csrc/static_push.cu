@@ -134,8 +134,8 @@ extern "C" psatd_status psatd_push_box_static(const int32_t n[3], int32_t order_
   const int64_t qtot = (int64_t)hx * (n1 / 2 + 1) * (n2 / 2 + 1);
   BoxDev b{};
   for (int a = 0; a < 3; ++a) b.n[a] = n[a];
-  b.scale64 = 1.0 / ((double)n0 * n1 * n2);
-  b.scale32 = (float)b.scale64;
+  s.scale64 = 1.0 / ((double)n0 * n1 * n2);
+  s.scale32 = (float)s.scale64;
   const int64_t spec = (int64_t)hx * n1 * n2;
   std::vector<RowJob> rows;
   std::vector<ColJob> ycols, zcols;
